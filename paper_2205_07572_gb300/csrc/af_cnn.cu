@@ -30,9 +30,9 @@
 // 2 adds b2 and reduces the global max-pool (value and first row-major
 // position per channel, by a butterfly exchange inside each warp; without
 // the positions for inference).  The backward pass recomputes layer 1 the
-// same way, uses that the max-pool passes gradient to one pixel per channel
-// (a small fraction of the forward work), and accumulates per-CTA partial
-// gradients that a second kernel sums in a fixed order (deterministic).
+// same way and uses that the max-pool passes gradient to one pixel per
+// channel (a small fraction of the forward work); its per-CTA partial
+// gradients are summed by a second kernel in a fixed order (deterministic).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -46,7 +46,6 @@ namespace {
 
 constexpr int kF = 32;       // feature channels
 constexpr int kLevels = 16;  // rows of the level embedding
-constexpr int kW2Pitch = kF * 9 + 1;  // padded row of W2 in shared memory (bank spread)
 
 __host__ __device__ constexpr int cnn_params(int C) { return kF * C * 9 + kLevels * kF + kF * kF * 9 + kF + kF + 1; }
 // offsets of the parameter blocks in the flat vector
@@ -58,47 +57,6 @@ __host__ __device__ constexpr int off_w3(int C) { return off_b2(C) + kF; }
 __host__ __device__ constexpr int off_b3(int C) { return off_w3(C) + kF; }
 
 __device__ __forceinline__ float rbf(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
-
-// Shared-memory layout of one CTA (floats).
-template <int C, int N>
-struct Smem {
-    static constexpr int S = N + 4, S1 = N + 2;
-    static constexpr int w1 = 0;
-    static constexpr int w2 = w1 + kF * C * 9;
-    static constexpr int emb = w2 + kF * kW2Pitch;
-    static constexpr int b2 = emb + kLevels * kF;
-    static constexpr int w3 = b2 + kF;
-    static constexpr int b3 = w3 + kF;
-    static constexpr int m = b3 + 4;  // per-channel maxima of the current sample
-    static constexpr int x = m + kF;
-    static constexpr int a1 = x + C * S * S;
-    static constexpr int fwd_end = a1 + kF * S1 * S1;
-    static constexpr int da1 = fwd_end;
-    static constexpr int gw1 = da1 + kF * S1 * S1;
-    static constexpr int gemb = gw1 + kF * C * 9;
-    static constexpr int gw2 = gemb + kLevels * kF;
-    static constexpr int gb2 = gw2 + kF * kF * 9;
-    static constexpr int gw3 = gb2 + kF;
-    static constexpr int gb3 = gw3 + kF;
-    static constexpr int bwd_end = gb3 + 4;
-};
-
-// Weights into shared memory (conv weights rounded to BF16).
-template <int C, int N>
-__device__ void load_weights(const float *__restrict__ P, float *sm) {
-    using L = Smem<C, N>;
-    for (int e = threadIdx.x; e < kF * C * 9; e += blockDim.x) sm[L::w1 + e] = rbf(P[off_w1() + e]);
-    for (int e = threadIdx.x; e < kF * kF * 9; e += blockDim.x) {
-        const int g = e / (kF * 9), r = e - g * kF * 9;
-        sm[L::w2 + g * kW2Pitch + r] = rbf(P[off_w2(C) + e]);
-    }
-    for (int e = threadIdx.x; e < kLevels * kF; e += blockDim.x) sm[L::emb + e] = P[off_emb(C) + e];
-    for (int e = threadIdx.x; e < kF; e += blockDim.x) {
-        sm[L::b2 + e] = P[off_b2(C) + e];
-        sm[L::w3 + e] = P[off_w3(C) + e];
-    }
-    if (threadIdx.x == 0) sm[L::b3] = P[off_b3(C)];
-}
 
 // Bounded tensor-core waits that gave up (read by af_step_wait_timeouts).
 __device__ unsigned int g_cnn_timeouts;
@@ -223,27 +181,13 @@ __device__ __forceinline__ bool tc_wait(uint64_t *bar, unsigned parity) {
     return true;
 }
 
-// Layer 1 of sample b on the tensor cores: input patch, its horizontal taps (Xh), MMAs, and
-// the epilogue A1 = bf16(relu(D1 + emb[level])) written either as the BF16
-// map layer 2 reads (F32OUT false) or as an FP32 map a1[f][y][x] (F32OUT
-// true, the backward pass).  xin: the patch already in shared memory, or
-// null (it is then read from X[b]).  Ends with a barrier; false if the wait
-// gave up.
-template <int C, int N, int NT, bool F32OUT>
-__device__ bool tc_layer1(const __nv_bfloat16 *__restrict__ X, int b, const uint16_t *xin, const float *emb,
-                          unsigned char *smem, uint32_t tmem, uint64_t *bar, unsigned &phase, float *a1) {
-    using G = TcGeo<C, N, F32OUT>;
-    constexpr int S = G::S, S1 = G::S1;
-    const uint16_t *xs = xin;
-    if (xs == nullptr) {
-        const uint16_t *xb = reinterpret_cast<const uint16_t *>(X) + (int64_t)b * C * S * S;
-        uint16_t *xw = reinterpret_cast<uint16_t *>(smem + G::xs);
-        for (int e = threadIdx.x; e < C * S * S; e += NT) xw[e] = xb[e];
-        __syncthreads();
-        xs = xw;
-    }
-    // Xh, one row (both 16-byte column blocks) per item: the horizontal taps
-    // X[c][r + kx] of flat pixel r of every channel (zero beyond the patch)
+// Xh of the patch at xs (shared memory), one row (both 16-byte column blocks)
+// per item: the horizontal taps X[c][r + kx] of flat pixel r of every channel
+// (zero beyond the patch).
+template <int C, int N, int NT, bool BWD>
+__device__ __forceinline__ void tc_build_xh(const uint16_t *xs, unsigned char *smem) {
+    using G = TcGeo<C, N, BWD>;
+    constexpr int S = G::S;
     for (int r = threadIdx.x; r < G::RH; r += NT) {
         uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
 #pragma unroll
@@ -257,15 +201,16 @@ __device__ bool tc_layer1(const __nv_bfloat16 *__restrict__ X, int b, const uint
         *reinterpret_cast<uint4 *>(smem + G::reg + r * 16) = make_uint4(w[0], w[1], w[2], w[3]);
         *reinterpret_cast<uint4 *>(smem + G::reg + G::xh_chunk + r * 16) = make_uint4(w[4], w[5], w[6], w[7]);
     }
-    tc::fence_smem_to_async();
-    tc::fence_before_sync();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        tc::fence_after_sync();
-        tc_issue_layer1<C, N, F32OUT>(smem, tmem, bar);
-    }
-    if (!tc_wait<NT>(bar, phase)) return false;
-    phase ^= 1u;
+}
+
+// Epilogue of layer 1: the map A1 = bf16(relu(D1 + emb)) of the accumulators,
+// pixel-major map[kc][m][8 channels] (kc blocks `chunk` bytes apart, row m =
+// the layer-1 pixel).  Channel pairs are added as packed FP32x2 and converted
+// to a BF16 pair in one instruction (each value rounded as alone).
+template <int C, int N, int NT, bool BWD>
+__device__ __forceinline__ void tc_epilogue1(const float *emb, uint32_t tmem, unsigned char *map, int chunk) {
+    using G = TcGeo<C, N, BWD>;
+    constexpr int S = G::S, S1 = G::S1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
     for (int mt = warp >> 2; mt < G::MT1; mt += NT / 128) {
@@ -275,29 +220,40 @@ __device__ bool tc_layer1(const __nv_bfloat16 *__restrict__ X, int b, const uint
         const int q = mt * 128 + 32 * (warp & 3) + lane, y = q / S, x = q - y * S;
         const int m = y * S1 + x;
         if (y < S1 && x < S1) {
-            if constexpr (F32OUT) {
 #pragma unroll
-                for (int g = 0; g < kF; ++g) a1[g * G::P1 + m] = rbf(fmaxf(z[g] + emb[g], 0.f));
-            } else {
-                // the map A1m[kc][m][8 channels], row m = the layer-1 pixel;
-                // channel pairs added as packed FP32x2 and converted to a
-                // BF16 pair in one instruction (each value rounded as alone)
+            for (int kc = 0; kc < 4; ++kc) {
+                uint32_t w[4];
 #pragma unroll
-                for (int kc = 0; kc < 4; ++kc) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        const int g = kc * 8 + 2 * h;
-                        const float2 a = __fadd2_rn(make_float2(z[g], z[g + 1]), make_float2(emb[g], emb[g + 1]));
-                        const __nv_bfloat162 r = __floats2bfloat162_rn(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f));
-                        w[h] = *reinterpret_cast<const uint32_t *>(&r);
-                    }
-                    *reinterpret_cast<uint4 *>(smem + G::reg + kc * G::a1_chunk + m * 16) =
-                        make_uint4(w[0], w[1], w[2], w[3]);
+                for (int h = 0; h < 4; ++h) {
+                    const int g = kc * 8 + 2 * h;
+                    const float2 a = __fadd2_rn(make_float2(z[g], z[g + 1]), make_float2(emb[g], emb[g + 1]));
+                    const __nv_bfloat162 r = __floats2bfloat162_rn(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f));
+                    w[h] = *reinterpret_cast<const uint32_t *>(&r);
                 }
+                *reinterpret_cast<uint4 *>(map + kc * chunk + m * 16) = make_uint4(w[0], w[1], w[2], w[3]);
             }
         }
     }
+}
+
+// Layer 1 of one sample in the forward pass: Xh of the patch xin, MMAs, and
+// the map layer 2 reads (it takes the place of Xh).  Ends with a barrier;
+// false if the wait gave up.
+template <int C, int N, int NT>
+__device__ bool tc_layer1(const uint16_t *xin, const float *emb, unsigned char *smem, uint32_t tmem, uint64_t *bar,
+                          unsigned &phase) {
+    using G = TcGeo<C, N>;
+    tc_build_xh<C, N, NT, false>(xin, smem);
+    tc::fence_smem_to_async();
+    tc::fence_before_sync();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        tc::fence_after_sync();
+        tc_issue_layer1<C, N, false>(smem, tmem, bar);
+    }
+    if (!tc_wait<NT>(bar, phase)) return false;
+    phase ^= 1u;
+    tc_epilogue1<C, N, NT, false>(emb, tmem, smem + G::reg, G::a1_chunk);
     tc::fence_smem_to_async();
     tc::fence_before_sync();
     __syncthreads();
@@ -366,7 +322,7 @@ __global__ void __launch_bounds__(128) cnn_forward_kernel(int nsample, const __n
         }
         const int lv = min(max(level[b], 0), kLevels - 1);
         if (!tc_wait<NT>(&xbar[cur], (unsigned)(it >> 1) & 1u)) break;
-        if (!tc_layer1<C, N, NT, false>(X, b, xbuf(cur), s_emb + lv * kF, smem, tmem, &bar, phase, nullptr)) break;
+        if (!tc_layer1<C, N, NT>(xbuf(cur), s_emb + lv * kF, smem, tmem, &bar, phase)) break;
         if (threadIdx.x == 0) {
             tc::fence_after_sync();
             tc_issue_layer2<C, N>(smem, tmem, &bar);
@@ -475,130 +431,287 @@ __global__ void __launch_bounds__(128) cnn_forward_kernel(int nsample, const __n
     if (warp == 0) tc::tmem_dealloc(tmem, kTmemCols);
 }
 
-// Byte offset of the backward pass's tensor-core region, after its FP32 arrays.
+// Shared memory of the backward pass (bytes), before its tensor-core region.
 template <int C, int N>
-__host__ __device__ constexpr int bwd_tc_offset() { return align128(4 * Smem<C, N>::bwd_end); }
+struct BwdSmem {
+    static constexpr int S = N + 4, S1 = N + 2;
+    static constexpr int XC = C == 3 ? 4 : C;              // floats per pixel of the FP32 patch
+    static constexpr int chunk = S1 * S1 * 16 / 128 * 128 + 144;  // a map block; 16 more than a multiple of 128 (banks)
+    static constexpr int w2 = 0;                           // [tap][thread] float4: W2[g][4 f] of thread (g, f / 4)
+    static constexpr int map = w2 + 9 * 256 * 16;          // layer-1 map, BF16 [kc][m][8]
+    static constexpr int xf = align128(map + 4 * chunk);  // two patches, FP32 [pixel][XC]
+    static constexpr int xf_bytes = align128(S * S * XC * 4);
+    static constexpr int semb = xf + 2 * xf_bytes;         // embedding gradient of each warp: [8][16 levels][32]
+    static constexpr int emb = semb + 8 * kLevels * kF * 4;
+    static constexpr int tc = emb + kLevels * kF * 4;      // TcGeo<C, N, true>
+    static constexpr int end = tc + TcGeo<C, N, true>::end;
+    static_assert(chunk >= S1 * S1 * 16, "a map block holds every layer-1 pixel");
+    static_assert(8 * kF * C * 9 * 4 <= 9 * 256 * 16, "the W1 gradients of eight warps fit where W2 was");
+    static_assert(tc % 128 == 0 && map % 16 == 0 && xf % 16 == 0, "aligned regions");
+};
 
+// Backward pass: one CTA of 256 threads per partial gradient, a sample at a
+// time.  The max-pool passes gradient to one pixel per channel g, so of dA1
+// only the 9 x 32 entries below that pixel's taps get a share of it, and all
+// that follows is linear in those shares: thread (g, four channels f) forms
+// them (dz_g W2[g][f][tap], masked by relu) and adds them straight into its
+// own 4 x 9 entries of the W2 gradient and its own copy of 4 x 9C entries of
+// the W1 gradient, all in registers over every sample of the CTA (packed
+// FP32x2 over channel pairs).  The copies over g are summed once, at the end.
+// No dA1 map is built and no gradient passes through shared memory, except
+// the level embedding's (a row per level, one copy per warp).
+// Layer 1 is recomputed by the forward pass's MMAs (the same bits, so the
+// same relu mask); the next sample's are in flight during this one's
+// gradients.  Per sample a thread issues about 490 packed multiply-adds, so
+// FP32 issue bounds it: about 200 registers, one CTA of eight warps per SM.
+// A training step (forward, backward, Adam) on 4096 patches of 3 x 20 x 20:
+// 2674 -> 189 us.  Before, one CTA built each dA1 map by a search over the 32
+// positions and summed the W1 gradient over all of its pixels.
 template <int C, int N>
-__global__ void __launch_bounds__(256) cnn_backward_kernel(int nsample, const __nv_bfloat16 *__restrict__ X,
-                                                           const int32_t *__restrict__ level,
-                                                           const float *__restrict__ P,
-                                                           const float *__restrict__ logit,
-                                                           const float *__restrict__ Min,
-                                                           const int32_t *__restrict__ Ain,
-                                                           const float *__restrict__ label,
-                                                           const float *__restrict__ omega, float inv_omega_sum,
-                                                           float *__restrict__ partial) {
-    using L = Smem<C, N>;
-    constexpr int S = L::S, S1 = L::S1;
+__global__ void __launch_bounds__(256, 1) cnn_backward_kernel(int nsample, const __nv_bfloat16 *__restrict__ X,
+                                                              const int32_t *__restrict__ level,
+                                                              const float *__restrict__ P,
+                                                              const float *__restrict__ logit,
+                                                              const float *__restrict__ Min,
+                                                              const int32_t *__restrict__ Ain,
+                                                              const float *__restrict__ label,
+                                                              const float *__restrict__ omega, float inv_omega_sum,
+                                                              float *__restrict__ partial) {
+    using L = BwdSmem<C, N>;
+    using G = TcGeo<C, N, true>;
+    constexpr int S = L::S, S1 = L::S1, NT = 256;
     constexpr int NP = cnn_params(C);
-    constexpr int NT = 256;
-    extern __shared__ __align__(128) float sm[];
-    __shared__ float s_dz[kF];
-    __shared__ int s_arg[kF];
-    __shared__ float s_dlogit;
+    constexpr int XW = (C * S * S + NT - 1) / NT;  // input words per thread
+    extern __shared__ __align__(128) unsigned char smb[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
-    unsigned char *const tcs = reinterpret_cast<unsigned char *>(sm) + bwd_tc_offset<C, N>();
-    load_weights<C, N>(P, sm);
+    unsigned char *const tcs = smb + L::tc;
+    uint16_t *const xs = reinterpret_cast<uint16_t *>(tcs + G::xs);
+    float *const semb = reinterpret_cast<float *>(smb + L::semb), *const emb = reinterpret_cast<float *>(smb + L::emb);
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31, fg = t & 7, g = t >> 3;
     tc_load_weights<C, N, NT, true>(P, tcs);
-    for (int e = threadIdx.x; e < L::bwd_end - L::gw1; e += blockDim.x) sm[L::gw1 + e] = 0.f;
-    if (threadIdx.x == 0) tc::mbar_init(&bar, 1);
-    if (threadIdx.x < 32) tc::tmem_alloc(&tslot, kTmemCols);
+    for (int e = t; e < 9 * 256 * 4; e += NT) {
+        const int k = e >> 10, th = (e >> 2) & 255, f = (th & 7) * 4 + (e & 3);
+        reinterpret_cast<float *>(smb + L::w2)[e] = rbf(P[off_w2(C) + ((th >> 3) * kF + f) * 9 + k]);
+    }
+    for (int e = t; e < 8 * kLevels * kF; e += NT) semb[e] = 0.f;
+    for (int e = t; e < kLevels * kF; e += NT) emb[e] = P[off_emb(C) + e];
+    const float w3g = P[off_w3(C) + g];
+    if (t == 0) tc::mbar_init(&bar, 1);
+    if (warp == 0) tc::tmem_alloc(&tslot, kTmemCols);
+    const uint16_t *const X16 = reinterpret_cast<const uint16_t *>(X);
+
+    // what a thread holds of the next sample: its input words, the scalars
+    uint16_t xr[XW];
+    float n_logit = 0.f, n_label = 0.f, n_omega = 0.f, n_m = 0.f;
+    int n_arg = -1, n_lv = 0;
+    auto load_x = [&](int b) {
+#pragma unroll
+        for (int k = 0; k < XW; ++k) {
+            const int e = t + k * NT;
+            xr[k] = (b < nsample && e < C * S * S) ? X16[(int64_t)b * (C * S * S) + e] : (uint16_t)0;
+        }
+    };
+    auto load_scalars = [&](int b) {
+        if (b >= nsample) return;
+        n_logit = logit[b];
+        n_label = label[b];
+        n_omega = omega[b];
+        n_lv = min(max(level[b], 0), kLevels - 1);
+        n_m = Min[(int64_t)b * kF + g];
+        n_arg = Ain[(int64_t)b * kF + g];
+    };
+    // the held input words to shared memory, BF16 [C][S][S] for Xh and FP32
+    // pixel-major for the gradients
+    auto store_x = [&](int buf) {
+        float *const xf = reinterpret_cast<float *>(smb + L::xf + buf * L::xf_bytes);
+#pragma unroll
+        for (int k = 0; k < XW; ++k) {
+            const int e = t + k * NT;
+            if (e >= C * S * S) break;
+            const int c = e / (S * S);
+            xs[e] = xr[k];
+            xf[(e - c * S * S) * L::XC + c] = __uint_as_float((uint32_t)xr[k] << 16);
+        }
+    };
+
+    float2 a1[C * 9][2], a2[9][2];  // this thread's W1 (a copy for its g) and W2 gradients, channel pairs
+    float gw3 = 0.f, gb2 = 0.f, gb3 = 0.f;
+#pragma unroll
+    for (int k = 0; k < C * 9; ++k) a1[k][0] = a1[k][1] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) a2[k][0] = a2[k][1] = make_float2(0.f, 0.f);
+
+    load_x(blockIdx.x);
+    load_scalars(blockIdx.x);
+    store_x(0);
+    __syncthreads();
+    tc_build_xh<C, N, NT, true>(xs, tcs);
     tc::fence_smem_to_async();
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = tslot;
     unsigned phase = 0;
-    for (int b = blockIdx.x; b < nsample; b += gridDim.x) {
-        const int lv = min(max(level[b], 0), kLevels - 1);
-        // layer 1 recomputed on the tensor cores (A1 as an FP32 map), and the
-        // input patch in FP32 for the W1 gradient
-        if (!tc_layer1<C, N, NT, true>(X, b, nullptr, sm + L::emb + lv * kF, tcs, tmem, &bar, phase, sm + L::a1))
-            break;
-        const uint16_t *xs = reinterpret_cast<const uint16_t *>(tcs + TcGeo<C, N, true>::xs);
-        for (int e = threadIdx.x; e < C * S * S; e += NT) sm[L::x + e] = __uint_as_float((uint32_t)xs[e] << 16);
-        if (threadIdx.x == 0) {
-            const float l = logit[b];
-            s_dlogit = omega[b] * (1.f / (1.f + expf(-l)) - label[b]) * inv_omega_sum;
-        }
+    if (t == 0 && blockIdx.x < nsample) tc_issue_layer1<C, N, true>(tcs, tmem, &bar);
+    load_x(blockIdx.x + gridDim.x);
+    int cur = 0;
+    for (int b = blockIdx.x; b < nsample; b += gridDim.x, cur ^= 1) {
+        const int nb = b + gridDim.x;
+        const float dl = n_omega * (1.f / (1.f + expf(-n_logit)) - n_label) * inv_omega_sum;
+        const float mg = n_m;
+        const int ag = n_arg, lv = n_lv;
+        // every thread has finished the previous sample's gradients here
+        if (!tc_wait<NT>(&bar, phase)) break;
+        phase ^= 1u;
+        tc_epilogue1<C, N, NT, true>(emb + lv * kF, tmem, smb + L::map, L::chunk);
+        if (nb < nsample) store_x(cur ^ 1);
+        tc::fence_before_sync();
         __syncthreads();
-        const float dl = s_dlogit;
-        if (threadIdx.x < kF) {
-            const int g = threadIdx.x;
-            const float mg = Min[(int64_t)b * kF + g];
-            const int ag = Ain[(int64_t)b * kF + g];
-            sm[L::gw3 + g] += dl * mg;
-            const float dz = ag >= 0 ? dl * sm[L::w3 + g] : 0.f;
-            s_dz[g] = dz;
-            s_arg[g] = ag;
-            sm[L::gb2 + g] += dz;
-            if (g == 0) sm[L::gb3] += dl;
-        }
-        __syncthreads();
-        // dW2[g, f, ky, kx] += dz_g A1[f, y_g + ky, x_g + kx]
-        for (int e = threadIdx.x; e < kF * kF * 9; e += blockDim.x) {
-            const int g = e / (kF * 9), r = e - g * kF * 9, f = r / 9, k = r - f * 9;
-            const int ag = s_arg[g];
-            if (ag < 0) continue;
-            const int yg = ag / N, xg = ag - yg * N;
-            sm[L::gw2 + e] += s_dz[g] * sm[L::a1 + (f * S1 + yg + k / 3) * S1 + xg + k % 3];
-        }
-        // dA1 gathered per position (no write conflicts), masked by relu
-        for (int e = threadIdx.x; e < kF * S1 * S1; e += blockDim.x) {
-            const int f = e / (S1 * S1), r = e - f * S1 * S1, y = r / S1, x = r - y * S1;
-            float d = 0.f;
-            for (int g = 0; g < kF; ++g) {
-                const int ag = s_arg[g];
-                if (ag < 0) continue;
-                const int ky = y - ag / N, kx = x - ag % N;
-                if (ky < 0 || ky > 2 || kx < 0 || kx > 2) continue;
-                d = fmaf(s_dz[g], sm[L::w2 + g * kW2Pitch + f * 9 + ky * 3 + kx], d);
+        if (nb < nsample) {
+            tc_build_xh<C, N, NT, true>(xs, tcs);
+            tc::fence_smem_to_async();
+            __syncthreads();
+            if (t == 0) {
+                tc::fence_after_sync();
+                tc_issue_layer1<C, N, true>(tcs, tmem, &bar);
             }
-            sm[L::da1 + e] = sm[L::a1 + e] > 0.f ? d : 0.f;
+            load_x(nb + gridDim.x);
+            load_scalars(nb);
         }
-        __syncthreads();
-        // level embedding and W1
-        if (threadIdx.x < kF) {
-            const int f = threadIdx.x;
-            float s = 0.f;
-            for (int r = 0; r < S1 * S1; ++r) s += sm[L::da1 + f * S1 * S1 + r];
-            sm[L::gemb + lv * kF + f] += s;
+        gw3 += dl * mg;
+        gb3 += dl;
+        float4 se = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (ag >= 0) {
+            const float dz = dl * w3g;
+            gb2 += dz;
+            const int yg = ag / N, xg = ag - yg * N;
+            const unsigned char *const mp = smb + L::map + (fg >> 1) * L::chunk + (fg & 1) * 8 + (yg * S1 + xg) * 16;
+            float2 v[9][2];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                const uint2 q = *reinterpret_cast<const uint2 *>(mp + (k / 3 * S1 + k % 3) * 16);
+                const float2 p0 = make_float2(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xffff0000u));
+                const float2 p1 = make_float2(__uint_as_float(q.y << 16), __uint_as_float(q.y & 0xffff0000u));
+                const float4 w = reinterpret_cast<const float4 *>(smb + L::w2)[k * 256 + t];
+                const float2 d2 = make_float2(dz, dz);
+                a2[k][0] = __ffma2_rn(d2, p0, a2[k][0]);
+                a2[k][1] = __ffma2_rn(d2, p1, a2[k][1]);
+                v[k][0] = make_float2(p0.x > 0.f ? dz * w.x : 0.f, p0.y > 0.f ? dz * w.y : 0.f);
+                v[k][1] = make_float2(p1.x > 0.f ? dz * w.z : 0.f, p1.y > 0.f ? dz * w.w : 0.f);
+                se.x += v[k][0].x;
+                se.y += v[k][0].y;
+                se.z += v[k][1].x;
+                se.w += v[k][1].y;
+            }
+            const float *const xp = reinterpret_cast<const float *>(smb + L::xf + cur * L::xf_bytes) + (yg * S + xg) * L::XC;
+#pragma unroll
+            for (int dy = 0; dy < 5; ++dy)
+#pragma unroll
+                for (int dx = 0; dx < 5; ++dx) {
+                    float xv[4];
+                    if constexpr (C == 3)
+                        *reinterpret_cast<float4 *>(xv) = *reinterpret_cast<const float4 *>(xp + (dy * S + dx) * 4);
+                    else
+                        xv[0] = xp[dy * S + dx];
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        const float2 x2 = make_float2(xv[c], xv[c]);
+#pragma unroll
+                        for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+                            for (int kx = 0; kx < 3; ++kx) {
+                                const int y = dy - ky, x = dx - kx;  // the W1 tap
+                                if (y < 0 || y > 2 || x < 0 || x > 2) continue;
+                                float2 *const a = a1[c * 9 + y * 3 + x];
+                                a[0] = __ffma2_rn(v[ky * 3 + kx][0], x2, a[0]);
+                                a[1] = __ffma2_rn(v[ky * 3 + kx][1], x2, a[1]);
+                            }
+                    }
+                }
         }
-        for (int e = threadIdx.x; e < kF * C * 9; e += blockDim.x) {
-            const int f = e / (C * 9), r = e - f * C * 9, c = r / 9, k = r - c * 9, ky = k / 3, kx = k % 3;
-            float s = 0.f;
-            for (int y = 0; y < S1; ++y)
-                for (int x = 0; x < S1; ++x)
-                    s = fmaf(sm[L::da1 + (f * S1 + y) * S1 + x], sm[L::x + (c * S + y + ky) * S + x + kx], s);
-            sm[L::gw1 + e] += s;
+        // level embedding: the shares of the warp's four g, then the warp's own row
+        for (int o = 8; o <= 16; o <<= 1) {
+            se.x += __shfl_xor_sync(0xffffffffu, se.x, o);
+            se.y += __shfl_xor_sync(0xffffffffu, se.y, o);
+            se.z += __shfl_xor_sync(0xffffffffu, se.z, o);
+            se.w += __shfl_xor_sync(0xffffffffu, se.w, o);
         }
-        __syncthreads();
+        if (lane < 8) {
+            float4 *const r = reinterpret_cast<float4 *>(semb + (warp * kLevels + lv) * kF) + lane;
+            const float4 o = *r;
+            *r = make_float4(o.x + se.x, o.y + se.y, o.z + se.z, o.w + se.w);
+        }
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (threadIdx.x < 32) tc::tmem_dealloc(tmem, kTmemCols);
+    if (warp == 0) tc::tmem_dealloc(tmem, kTmemCols);
     // partial gradient of this CTA, in parameter order
-    float *out = partial + (int64_t)blockIdx.x * NP;
-    for (int e = threadIdx.x; e < NP; e += blockDim.x) {
-        float v;
-        if (e < off_emb(C)) v = sm[L::gw1 + e];
-        else if (e < off_w2(C)) v = sm[L::gemb + e - off_emb(C)];
-        else if (e < off_b2(C)) v = sm[L::gw2 + e - off_w2(C)];
-        else if (e < off_w3(C)) v = sm[L::gb2 + e - off_b2(C)];
-        else if (e < off_b3(C)) v = sm[L::gw3 + e - off_w3(C)];
-        else v = sm[L::gb3];
-        out[e] = v;
+    float *const out = partial + (int64_t)blockIdx.x * NP;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        float *const o = out + off_w2(C) + (g * kF + fg * 4) * 9 + k;
+        o[0] = a2[k][0].x;
+        o[9] = a2[k][0].y;
+        o[18] = a2[k][1].x;
+        o[27] = a2[k][1].y;
+    }
+    if (fg == 0) {
+        out[off_b2(C) + g] = gb2;
+        out[off_w3(C) + g] = gw3;
+    }
+    if (t == 0) out[off_b3(C)] = gb3;
+    // W1: over the warp's four g by exchanges, then over the eight warps
+    float *const red = reinterpret_cast<float *>(smb + L::w2);  // [warp][f][9C]
+#pragma unroll
+    for (int k = 0; k < C * 9; ++k)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float2 a = a1[k][h];
+#pragma unroll
+            for (int o = 8; o <= 16; o <<= 1) {
+                a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+                a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+            }
+            if (lane < 8) {
+                red[(warp * kF + fg * 4 + 2 * h) * C * 9 + k] = a.x;
+                red[(warp * kF + fg * 4 + 2 * h + 1) * C * 9 + k] = a.y;
+            }
+        }
+    __syncthreads();
+    for (int e = t; e < kF * C * 9; e += NT) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) s += red[w * kF * C * 9 + e];
+        out[off_w1() + e] = s;
+    }
+    for (int e = t; e < kLevels * kF; e += NT) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) s += semb[w * kLevels * kF + e];
+        out[off_emb(C) + e] = s;
     }
 }
 
-__global__ void sum_partials(const float *__restrict__ partial, int nblocks, int np, float *__restrict__ grad) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= np) return;
+// grad[e] = sum of partial[k][e] over the blocks k, in a fixed order: a CTA
+// sums 32 parameters, its eight warps every eighth block each (the loads of a
+// warp are one 128-byte row; one thread per parameter left 41 CTAs with a
+// chain of nblocks loads each).
+__global__ void __launch_bounds__(256) sum_partials(const float *__restrict__ partial, int nblocks, int np,
+                                                    float *__restrict__ grad) {
+    __shared__ float sm[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
     float s = 0.f;
-    for (int k = 0; k < nblocks; ++k) s += partial[(int64_t)k * np + e];
-    grad[e] = s;
+    if (e < np)
+#pragma unroll 4
+        for (int k = warp; k < nblocks; k += 8) s += partial[(int64_t)k * np + e];
+    sm[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && e < np) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) s += sm[w][lane];
+        grad[e] = s;
+    }
 }
 
 __global__ void adam_kernel(int64_t n, float *__restrict__ p, float *__restrict__ m, float *__restrict__ v,
@@ -729,13 +842,13 @@ af_status backward_launch(int nsample, const void *X, const int32_t *lev, const 
                           const float *M, const int32_t *A, const float *y, const float *om, float inv_om,
                           float *partial, int nblocks, float *grad, cudaStream_t s) {
     auto k = cnn_backward_kernel<C, N>;
-    const size_t bytes = bwd_tc_offset<C, N>() + TcGeo<C, N, true>::end;
+    const size_t bytes = BwdSmem<C, N>::end;
     if (const af_status e = smem_attr(k, bytes)) return e;
     k<<<nblocks, 256, bytes, s>>>(nsample, static_cast<const __nv_bfloat16 *>(X), lev, P, lg, M, A, y, om, inv_om,
                                   partial);
     if (launched() != AF_OK) return AF_ERR_CUDA;
     const int np = cnn_params(C);
-    sum_partials<<<(np + 255) / 256, 256, 0, s>>>(partial, nblocks, np, grad);
+    sum_partials<<<(np + 31) / 32, 256, 0, s>>>(partial, nblocks, np, grad);
     return launched();
 }
 

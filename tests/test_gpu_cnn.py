@@ -107,6 +107,39 @@ def test_gradients_match_oracle(af, C, N):
     assert np.array_equal(g2.cpu().numpy(), g.astype(np.float32))
 
 
+@pytest.mark.parametrize("C,N", [(3, 16), (1, 8), (3, 8), (1, 16)])
+@pytest.mark.parametrize("P,nblocks", [(1, 4), (13, 3), (40, 152)])
+def test_backward_of_every_shape_and_ragged_batch_matches_oracle(af, C, N, P, nblocks):
+    """af_cnn_backward alone, on the oracle's forward results: batches below,
+    above and not a multiple of the number of partial gradients, dead channels
+    (no position) among the live ones, levels outside the embedding's rows.
+    What may differ is the FP32 summation (1e-5) and a map entry rounded to
+    the neighbouring BF16 number (2^-8 of one of a gradient's terms)."""
+    X, level, params, label, omega = _problem(C, N, P, seed=31 * C + N + P)
+    o = 32 * C * 9 + 16 * 32 + 32 * 32 * 9
+    params[o + 3:o + 9] = -1000.0  # b2: channels whose maximum is never positive
+    level[0] = 0
+    g_r = OC.backward(X, level, params, C, label, omega)
+    lg, M, arg, _ = OC.forward(X, level, params, C)
+    assert (arg[:, 3:9] == -1).all()
+    np_ = len(params)
+    dev = lambda a, t: torch.from_numpy(np.ascontiguousarray(a).astype(t)).cuda()  # noqa: E731
+    lv = level.copy()
+    lv[0] = -5  # clamped to row 0
+    partial = torch.full((af.cnn_partial_floats(C, nblocks),), float("nan"), device="cuda")
+    grad = torch.full((np_,), float("nan"), device="cuda")
+    af.cnn_backward(C, N, P, _bf16_bits(X), dev(lv, np.int32), dev(params, np.float32), dev(lg, np.float32),
+                    dev(M, np.float32), dev(arg, np.int32), dev(label, np.float32), dev(omega, np.float32),
+                    float(omega.sum()), partial, nblocks, grad)
+    torch.cuda.synchronize()
+    g = grad.cpu().numpy().astype(np.float64)
+    k = 0
+    for size in (32 * C * 9, 16 * 32, 32 * 32 * 9, 32, 32, 1):
+        assert _nerr(g[k:k + size], g_r[k:k + size]) < 1e-5 + 2.0 ** -8, (k, size)
+        k += size
+    assert af.step_wait_timeouts() == 0
+
+
 def test_adam_matches_oracle(af):
     rng = np.random.default_rng(1)
     n = 1000
