@@ -74,6 +74,32 @@ def test_every_tiling_matches_oracle(af, field):
         assert _nerr(og, orf) < 1e-12, (k, tilings[k])
 
 
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,px,cfl", [(5, 1, 1.0), (2, 3, 1.0), (8, 3, 0.9), (16, 2, 1.0), (33, 2, 0.45), (64, 1, 1.0),
+                                      (8, 20, 1.0), (16, 12, 0.3)])
+def test_feet_of_every_displacement_match_oracle(af, n, px, cfl, prec):
+    """One swirl step with displacements from a fifth of the domain (CFL 1 on a
+    5 x 5 grid: the general turn) to a thousandth of it (the shortest series),
+    to the largest step the CFL condition allows, on tiles with and without
+    bulk staging.  A foot's error of eps dx moves a value by eps: the bounds of
+    one step hold."""
+    from paper_2205_07572_gb300.uniform import UniformRun
+    grid = S.UniformGrid(S.Layout(n, 1), px, px)
+    st = S.periodic_state(grid, [lambda x, y: np.sin(2 * np.pi * x) * np.cos(4 * np.pi * y) + 0.3 * np.cos(2 * np.pi * (x + y))],
+                          nq=3)
+    if prec:
+        st = st.astype(np.float32).astype(np.float64)
+    dt = cfl * grid.dx
+    vc = O.VarCfg(n, 1, grid.dx, grid.dy, dt, 0.0, 0.0, 0.1)
+    ref = O.run_uniform_var(vc, px, px, (0.0, 0.0), 1, st)
+    run = UniformRun(af.config(af.ADVECTION, prec, n), px, px, grid.dx, grid.dy, dt, state=st, field=af.FIELD_SWIRL, t0=0.1)
+    run.step()
+    torch.cuda.synchronize()
+    got = run.state.double().cpu().numpy().reshape(st.shape)
+    assert _nerr(S.unpack_owned(grid, got), S.unpack_owned(grid, ref)) < TOL[prec]
+    assert af.step_wait_timeouts() == 0
+
+
 @pytest.mark.parametrize("field", [0, 1])
 def test_constant_state_preserved_on_gpu(af, field):
     """Remark of Section 4.2 / Theorem of Section 4.3, FP64 on the GPU."""
