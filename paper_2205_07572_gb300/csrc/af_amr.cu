@@ -5,6 +5,10 @@
 // lmax, so a level-l cell is 2^(lmax-l+1) units wide and every node, cell
 // centre and Simpson point is a lattice point of that unit.  The forest is
 // located through per-level region maps (af_forest.d_map), which stay in L2.
+// They are 32-bit: the domain is (B << lmax) 2n units wide, and a map of
+// (B << lmax)^2 entries that fits the GPU keeps that below 2^25.  (With 64-bit
+// positions the divisions by a region's width were most of the kernels that
+// look owners up: on 2100 leaves a ghost plan took 209 us, now 69.)
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -17,7 +21,8 @@ namespace {
 struct DevForest {
     int nleaf, B, lmax, n;
     const int32_t *level, *ix, *iy, *map;
-    long long D;  // domain width in units
+    int D;           // domain width in units
+    uint32_t rcp;    // 2^32 / (2n) rounded up: region() divides by 2n with it
 };
 
 DevForest make_dev(const af_forest &f, int n) {
@@ -30,7 +35,8 @@ DevForest make_dev(const af_forest &f, int n) {
     d.ix = f.d_ix;
     d.iy = f.d_iy;
     d.map = f.d_map;
-    d.D = (long long)f.B * n * (2LL << f.lmax);
+    d.D = (int)((long long)f.B * n * (2LL << f.lmax));
+    d.rcp = (uint32_t)(((1ull << 32) + 2 * n - 1) / (2 * n));
     return d;
 }
 
@@ -39,49 +45,54 @@ __host__ __device__ inline long long map_offset(int B, int l) {
     return (long long)B * B * (((1LL << (2 * l)) - 1) / 3);
 }
 
-__device__ __forceinline__ long long hwid(const DevForest &F, int l) { return 2LL << (F.lmax - l); }
+// Width of a level-l cell in units.
+__device__ __forceinline__ int hwid(const DevForest &F, int l) { return 2 << (F.lmax - l); }
 
-__device__ __forceinline__ long long wrapd(const DevForest &F, long long x) {
+__device__ __forceinline__ int wrapd(const DevForest &F, int x) {
     // positions are at most one domain width outside [0, D)
-    if (x >= 0 && x < F.D) return x;
-    if (x < 0 && x >= -F.D) return x + F.D;
-    if (x >= F.D && x < 2 * F.D) return x - F.D;
-    long long r = x % F.D;
-    return r < 0 ? r + F.D : r;
+    if (x < 0) x += F.D;
+    if (x >= F.D) x -= F.D;
+    if ((unsigned)x >= (unsigned)F.D) {
+        x %= F.D;
+        return x < 0 ? x + F.D : x;
+    }
+    return x;
+}
+
+// Finest-level region (column or row) of position x >= 0: x / (2n).  The
+// product with the rounded-up reciprocal is too large by at most one.
+__device__ __forceinline__ int region(const DevForest &F, int x) {
+    const int q = (int)__umulhi((uint32_t)x, F.rcp);
+    return q * 2 * F.n > x ? q - 1 : q;
 }
 
 // Leaf whose half-open extent contains (x, y).  A region of the finest level
 // lmax is a leaf (entry q >= 0) or lies inside the coarser leaf -2 - entry
 // (af_forest_build_map), so one load finds it; a map without that second
 // kind of entry is searched level by level.
-__device__ int lookup(const DevForest &F, long long x, long long y) {
-    x = wrapd(F, x);
-    y = wrapd(F, y);
-    {
-        const long long pw = 2LL * F.n;  // a finest-level region, in units
-        const long long side = (long long)F.B << F.lmax;
-        const int q = __ldg(F.map + map_offset(F.B, F.lmax) + (y / pw) * side + (x / pw));
+__device__ __forceinline__ int lookup(const DevForest &F, int x, int y) {
+    const int rx = region(F, wrapd(F, x)), ry = region(F, wrapd(F, y));
+#pragma unroll 1
+    for (int l = F.lmax; l >= 0; --l) {
+        const int sh = F.lmax - l;
+        const int q = __ldg(F.map + map_offset(F.B, l) + (int64_t)(ry >> sh) * (F.B << l) + (rx >> sh));
         if (q >= 0) return q < F.nleaf ? q : -1;
-        if (q <= -2) return -2 - q < F.nleaf ? -2 - q : -1;
-    }
-    for (int l = F.lmax - 1; l >= 0; --l) {
-        const long long pw = (long long)F.n * hwid(F, l);
-        const long long side = (long long)F.B << l;
-        const int q = __ldg(F.map + map_offset(F.B, l) + (y / pw) * side + (x / pw));
-        if (q >= 0) return q < F.nleaf ? q : -1;
+        if (q <= -2 && l == F.lmax) return -2 - q < F.nleaf ? -2 - q : -1;
     }
     return -1;
 }
 
 // Owner of a point value: the finest leaf touching the point, ties in the
 // order above-right, above-left, below-right, below-left.
-__device__ int node_owner(const DevForest &F, long long x, long long y) {
-    int best = lookup(F, x, y);
-    int bl = best >= 0 ? __ldg(F.level + best) : -1;
-    const long long dx[3] = {-1, 0, -1}, dy[3] = {0, -1, -1};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const int q = lookup(F, x + dx[k], y + dy[k]);
+__device__ __forceinline__ int entry_owner(const DevForest &F, int plane, int x, int y) {
+    const int touching = plane == kAvg ? 1 : 4;  // an average's owner is the leaf around it
+    int best = -1, bl = -1;
+    // a loop, not four copies of lookup(): the callers' code has to stay small
+    // (unrolled everywhere, a regrid's transfer spent 25 of 32 cycles per
+    // instruction waiting for the instruction cache)
+#pragma unroll 1
+    for (int k = 0; k < touching; ++k) {
+        const int q = lookup(F, x - (k & 1), y - (k >> 1));
         if (q >= 0) {
             const int lq = __ldg(F.level + q);
             if (lq > bl) {
@@ -93,20 +104,16 @@ __device__ int node_owner(const DevForest &F, long long x, long long y) {
     return best;
 }
 
-__device__ __forceinline__ int entry_owner(const DevForest &F, int plane, long long x, long long y) {
-    return plane == kAvg ? lookup(F, x, y) : node_owner(F, x, y);
+__device__ __forceinline__ int leaf_x0(const DevForest &F, int q) {
+    return __ldg(F.ix + q) * F.n * hwid(F, __ldg(F.level + q));
 }
-
-__device__ __forceinline__ long long leaf_x0(const DevForest &F, int q) {
-    return (long long)__ldg(F.ix + q) * F.n * hwid(F, __ldg(F.level + q));
-}
-__device__ __forceinline__ long long leaf_y0(const DevForest &F, int q) {
-    return (long long)__ldg(F.iy + q) * F.n * hwid(F, __ldg(F.level + q));
+__device__ __forceinline__ int leaf_y0(const DevForest &F, int q) {
+    return __ldg(F.iy + q) * F.n * hwid(F, __ldg(F.level + q));
 }
 
 // x - x0 unwrapped across the periodic box
-__device__ __forceinline__ long long reld(const DevForest &F, long long x, long long x0) {
-    long long d = wrapd(F, x - x0);
+__device__ __forceinline__ int reld(const DevForest &F, int x, int x0) {
+    const int d = wrapd(F, x - x0);
     return d > F.D / 2 ? d - F.D : d;
 }
 
@@ -132,15 +139,14 @@ struct StateView {
 };
 
 // Lattice indices (i, j) of point (x, y) in plane k of leaf q.
-__device__ __forceinline__ void lattice_of(const DevForest &F, int q, int k, long long x, long long y, int &i,
-                                           int &j) {
+__device__ __forceinline__ void lattice_of(const DevForest &F, int q, int k, int x, int y, int &i, int &j) {
     const int sh = F.lmax - __ldg(F.level + q) + 1;  // hw = 2^sh
-    const long long hw = 1LL << sh;
-    long long dx = reld(F, x, leaf_x0(F, q)), dy = reld(F, y, leaf_y0(F, q));
+    const int hw = 1 << sh;
+    int dx = reld(F, x, leaf_x0(F, q)), dy = reld(F, y, leaf_y0(F, q));
     if (k == kAvg || k == kYmid) dx -= hw / 2;
     if (k == kAvg || k == kXmid) dy -= hw / 2;
-    i = (int)(dx >> sh);  // floor division (arithmetic shift)
-    j = (int)(dy >> sh);
+    i = dx >> sh;  // floor division (arithmetic shift)
+    j = dy >> sh;
     // owners are always within two cells of the lattice; clamp defensively
     const int lo = -kGhost, hi = F.n + kGhost;
     i = i < lo ? lo : (i > hi ? hi : i);
@@ -215,10 +221,14 @@ template <typename R, typename Fn>
 __device__ __forceinline__ R simpson9(Fn f) {
     const R w[3] = {R(1) / R(6), R(2) / R(3), R(1) / R(6)};
     R s = R(0);
-    for (int b = 0; b < 3; ++b)
-        for (int a = 0; a < 3; ++a) s = r_fma(r_mul(w[a], w[b]), f(a, b), s);
+#pragma unroll 1
+    for (int e = 0; e < 9; ++e) s = r_fma(r_mul(w[e % 3], w[e / 3]), f(e % 3, e / 3), s);
     return s;
 }
+
+// 2^-sh (exact)
+__device__ __forceinline__ void pow2_neg(int sh, float &r) { r = __int_as_float((127 - sh) << 23); }
+__device__ __forceinline__ void pow2_neg(int sh, double &r) { r = __longlong_as_double((long long)(1023 - sh) << 52); }
 
 // The nine values the reconstruction of one cell of leaf q combines at
 // (x, y) (component 0; component c is cstride entries further), and where
@@ -230,44 +240,45 @@ struct ReconSite {
     int qx, qy;     // quarter holding (x, y)
 };
 
+// Point value (plane k, lattice entry (ii, jj)) of leaf q, whose cells are hw
+// wide and whose corner is (x0, y0), component 0.  Point values on the leaf's
+// boundary lines are read from their owner: a leaf whose neighbours are all
+// same-level does not keep the copies in its ghost ring current (its step
+// reads the neighbours directly).
 template <typename T>
-__device__ void recon_locate(const DevForest &F, const StateView<T> &S, int q, long long x, long long y,
-                             ReconSite<T> &r) {
-    const int sh = F.lmax - __ldg(F.level + q) + 1;  // hw = 2^sh
-    const long long hw = 1LL << sh;
-    const long long dx = reld(F, x, leaf_x0(F, q)), dy = reld(F, y, leaf_y0(F, q));
-    long long ci = dx >= 0 ? (dx >> sh) : -1, cj = dy >= 0 ? (dy >> sh) : -1;
-    ci = ci < 0 ? 0 : (ci > F.n - 1 ? F.n - 1 : ci);
-    cj = cj < 0 ? 0 : (cj > F.n - 1 ? F.n - 1 : cj);
-    r.xi = (T)(2.0 * (double)(dx - ci * hw) / (double)hw - 1.0);  // exact: a multiple of 1/2
-    r.eta = (T)(2.0 * (double)(dy - cj * hw) / (double)hw - 1.0);
-    r.qx = 2 * (dx - ci * hw) >= hw;
-    r.qy = 2 * (dy - cj * hw) >= hw;
-    const int i = (int)ci, j = (int)cj;
-    // Point values on the leaf's boundary lines are read from their owner:
-    // a leaf whose neighbours are all same-level does not keep the copies in
-    // its ghost ring current (its step reads the neighbours directly).
-    auto node = [&](int k, int ii, int jj) -> const T * {
-        if (ii > 0 && ii < F.n && jj > 0 && jj < F.n) return S.at(q, 0, k, ii, jj);
-        const long long x0 = leaf_x0(F, q), y0 = leaf_y0(F, q);
-        const long long nx = x0 + (long long)ii * hw + (k == kYmid ? hw / 2 : 0);
-        const long long ny = y0 + (long long)jj * hw + (k == kXmid ? hw / 2 : 0);
-        const int o = node_owner(F, nx, ny);
-        if (o < 0 || o == q) return S.at(q, 0, k, ii, jj);
-        const int lo = __ldg(F.level + o);
-        const int ko = lo == __ldg(F.level + q) ? k : kCorner;
-        int oi, oj;
-        lattice_of(F, o, ko, nx, ny, oi, oj);
-        return S.at(o, 0, ko, oi, oj);
-    };
-    r.v[0] = node(kCorner, i, j);
-    r.v[1] = node(kCorner, i + 1, j);
-    r.v[2] = node(kCorner, i, j + 1);
-    r.v[3] = node(kCorner, i + 1, j + 1);
-    r.v[4] = node(kXmid, i, j);
-    r.v[5] = node(kXmid, i + 1, j);
-    r.v[6] = node(kYmid, i, j);
-    r.v[7] = node(kYmid, i, j + 1);
+__device__ __forceinline__ const T *node_value(const DevForest &F, const StateView<T> &S, int q, int lq, int x0, int y0,
+                                               int hw, int k, int ii, int jj) {
+    if (ii > 0 && ii < F.n && jj > 0 && jj < F.n) return S.at(q, 0, k, ii, jj);
+    const int nx = x0 + ii * hw + (k == kYmid ? hw / 2 : 0);
+    const int ny = y0 + jj * hw + (k == kXmid ? hw / 2 : 0);
+    const int o = entry_owner(F, k, nx, ny);
+    if (o < 0 || o == q) return S.at(q, 0, k, ii, jj);
+    const int lo = __ldg(F.level + o);
+    const int ko = lo == lq ? k : kCorner;
+    int oi, oj;
+    lattice_of(F, o, ko, nx, ny, oi, oj);
+    return S.at(o, 0, ko, oi, oj);
+}
+
+template <typename T>
+__device__ void recon_locate(const DevForest &F, const StateView<T> &S, int q, int x, int y, ReconSite<T> &r) {
+    const int lq = __ldg(F.level + q), sh = F.lmax - lq + 1;  // hw = 2^sh
+    const int hw = 1 << sh;
+    const int x0 = __ldg(F.ix + q) * F.n * hw, y0 = __ldg(F.iy + q) * F.n * hw;
+    const int dx = reld(F, x, x0), dy = reld(F, y, y0);
+    int i = dx >= 0 ? (dx >> sh) : 0, j = dy >= 0 ? (dy >> sh) : 0;
+    i = i > F.n - 1 ? F.n - 1 : i;
+    j = j > F.n - 1 ? F.n - 1 : j;
+    T rhw;
+    pow2_neg(sh, rhw);
+    r.xi = (T)(2 * (dx - i * hw) - hw) * rhw;  // exact: a multiple of 1/2 (of 2^-sh, below 2^24 units)
+    r.eta = (T)(2 * (dy - j * hw) - hw) * rhw;
+    r.qx = 2 * (dx - i * hw) >= hw;
+    r.qy = 2 * (dy - j * hw) >= hw;
+    auto node = [&](int k, int ii, int jj) { return node_value<T>(F, S, q, lq, x0, y0, hw, k, ii, jj); };
+#pragma unroll 1
+    for (int e = 0; e < 8; ++e)  // four corners, xl, xr, yb, yt
+        r.v[e] = node(e < 4 ? kCorner : (e < 6 ? kXmid : kYmid), i + (e < 6 ? e & 1 : 0), j + (e < 4 ? e >> 1 : (e == 7)));
     r.v[8] = S.at(q, 0, kAvg, i, j);
 }
 
@@ -286,53 +297,19 @@ __device__ __forceinline__ T recon_value(const ReconSite<T> &r, int64_t coff, bo
 // quarter set instead the mean of the reconstruction over the quarter of the
 // cell holding (x, y) that (x, y) lies in (the centre of a finer cell).
 template <typename T>
-__device__ T recon_at(const DevForest &F, const StateView<T> &S, int q, int c, long long x, long long y,
-                      bool quarter = false) {
+__device__ T recon_at(const DevForest &F, const StateView<T> &S, int q, int c, int x, int y, bool quarter = false) {
     ReconSite<T> r;
     recon_locate<T>(F, S, q, x, y, r);
     return recon_value<T>(r, (int64_t)c * kPlanes * S.plane, quarter);
 }
 
-// Value for an entry of plane k of a destination at level lp from owner q
-// (Section 3.1: copy, fine -> coarse, coarse -> fine).
+// Values of every component c < nc for an entry of plane k of a destination at
+// level lp from owner q (Section 3.1: copy, fine -> coarse, coarse -> fine).
+// Averages from finer cells are summed in FP64; what is copied or interpolated
+// stays in the state's precision.
 template <typename T>
-__device__ double transfer(const DevForest &F, const StateView<T> &S, int lp, int q, int c, int k, long long x,
-                           long long y) {
-    const int lq = __ldg(F.level + q);
-    int i, j;
-    if (lq == lp) {
-        lattice_of(F, q, k, x, y, i, j);
-        return *S.at(q, c, k, i, j);
-    }
-    if (lq > lp) {
-        if (k == kAvg) {
-            const long long h = hwid(F, lq) / 2;
-            double s = 0.0;
-#pragma unroll
-            for (int b = -1; b <= 1; b += 2)
-#pragma unroll
-                for (int a = -1; a <= 1; a += 2) {
-                    lattice_of(F, q, kAvg, x + a * h, y + b * h, i, j);
-                    s += *S.at(q, c, kAvg, i, j);
-                }
-            return 0.25 * s;
-        }
-        lattice_of(F, q, kCorner, x, y, i, j);
-        return *S.at(q, c, kCorner, i, j);
-    }
-    if (k != kAvg) return (double)recon_at<T>(F, S, q, c, x, y);
-    // the mean of the coarse biquadratic over the destination cell, a quarter
-    // of a coarse cell (the Simpson rule over it, exact for the biquadratic)
-    if (lq == lp - 1) return (double)recon_at<T>(F, S, q, c, x, y, true);
-    const long long h = hwid(F, lp) / 2;
-    return (double)simpson9<T>([&](int a, int b) { return recon_at<T>(F, S, q, c, x + (a - 1) * h, y + (b - 1) * h); });
-}
-
-// transfer() for every component c < nc at once (the owner's sites are
-// located once): out[c].
-template <typename T>
-__device__ void transfer_all(const DevForest &F, const StateView<T> &S, int lp, int q, int k, long long x,
-                             long long y, int nc, double out[3]) {
+__device__ void transfer_all(const DevForest &F, const StateView<T> &S, int lp, int q, int k, int x, int y, int nc,
+                             T out[3]) {
     const int lq = __ldg(F.level + q);
     const int64_t cs = (int64_t)kPlanes * S.plane;
     int i, j;
@@ -340,11 +317,11 @@ __device__ void transfer_all(const DevForest &F, const StateView<T> &S, int lp, 
         const int ko = lq == lp ? k : kCorner;
         lattice_of(F, q, ko, x, y, i, j);
         const T *v = S.at(q, 0, ko, i, j);
-        for (int c = 0; c < nc; ++c) out[c] = (double)v[c * cs];
+        for (int c = 0; c < nc; ++c) out[c] = v[c * cs];
         return;
     }
     if (lq > lp) {  // an average from a finer owner: the mean of its four cells
-        const long long h = hwid(F, lq) / 2;
+        const int h = hwid(F, lq) / 2;
         const T *v[4];
 #pragma unroll
         for (int b = 0; b < 2; ++b)
@@ -354,48 +331,62 @@ __device__ void transfer_all(const DevForest &F, const StateView<T> &S, int lp, 
                 v[2 * b + a] = S.at(q, 0, kAvg, i, j);
             }
         for (int c = 0; c < nc; ++c) {
-            // the same order of additions as transfer()
             double s = 0.0;
             s += (double)v[0][c * cs];
             s += (double)v[1][c * cs];
             s += (double)v[2][c * cs];
             s += (double)v[3][c * cs];
-            out[c] = 0.25 * s;
+            out[c] = (T)(0.25 * s);
         }
         return;
     }
     if (k != kAvg || lq == lp - 1) {  // a coarser owner: its reconstruction (quarter mean for an average)
         ReconSite<T> r;
         recon_locate<T>(F, S, q, x, y, r);
-        for (int c = 0; c < nc; ++c) out[c] = (double)recon_value<T>(r, c * cs, k == kAvg);
+        for (int c = 0; c < nc; ++c) out[c] = recon_value<T>(r, c * cs, k == kAvg);
         return;
     }
-    for (int c = 0; c < nc; ++c) out[c] = transfer<T>(F, S, lp, q, c, k, x, y);
+    // an average from an owner two or more levels coarser (a forest that is
+    // not 2:1 balanced): Simpson's rule over the destination cell
+    const int h = hwid(F, lp) / 2;
+    for (int c = 0; c < nc; ++c)
+        out[c] = simpson9<T>([&](int a, int b) { return recon_at<T>(F, S, q, c, x + (a - 1) * h, y + (b - 1) * h); });
 }
 
-__device__ __forceinline__ void entry_xy(const DevForest &F, int p, int k, int i, int j, long long &x, long long &y) {
-    const long long hw = hwid(F, __ldg(F.level + p));
-    x = leaf_x0(F, p) + (long long)i * hw + ((k == kAvg || k == kYmid) ? hw / 2 : 0);
-    y = leaf_y0(F, p) + (long long)j * hw + ((k == kAvg || k == kXmid) ? hw / 2 : 0);
+// transfer_all out of line: for the few entries of a leaf that need it.
+template <typename T>
+__device__ __noinline__ void transfer_entry(const DevForest &F, const StateView<T> &S, int lp, int q, int k, int x, int y,
+                                            T out[3]) {
+    transfer_all<T>(F, S, lp, q, k, x, y, S.ncomp, out);
+}
+
+__device__ __forceinline__ void entry_xy(const DevForest &F, int p, int k, int i, int j, int &x, int &y) {
+    const int hw = hwid(F, __ldg(F.level + p));
+    x = leaf_x0(F, p) + i * hw + ((k == kAvg || k == kYmid) ? hw / 2 : 0);
+    y = leaf_y0(F, p) + j * hw + ((k == kAvg || k == kXmid) ? hw / 2 : 0);
 }
 
 // True if some neighbour region of leaf p at its own level is not a leaf.
 __device__ bool has_other_level_neighbour(const DevForest &F, int p) {
     const int l = __ldg(F.level + p);
-    const long long side = (long long)F.B << l;
-    const long long px = __ldg(F.ix + p), py = __ldg(F.iy + p);
-    for (int sy = -1; sy <= 1; ++sy)
-        for (int sx = -1; sx <= 1; ++sx) {
-            if (sx == 0 && sy == 0) continue;
-            const long long nx = ((px + sx) % side + side) % side, ny = ((py + sy) % side + side) % side;
-            if (__ldg(F.map + map_offset(F.B, l) + ny * side + nx) < 0) return true;
-        }
-    return false;
+    const int side = F.B << l;
+    const int px = __ldg(F.ix + p), py = __ldg(F.iy + p);
+    const int32_t *const map = F.map + map_offset(F.B, l);
+    bool other = false;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        if (e == 4) continue;
+        int nx = px + e % 3 - 1, ny = py + e / 3 - 1;
+        nx = nx < 0 ? nx + side : (nx >= side ? nx - side : nx);
+        ny = ny < 0 ? ny + side : (ny >= side ? ny - side : ny);
+        other |= __ldg(map + (int64_t)ny * side + nx) < 0;
+    }
+    return other;
 }
 
 // One pass of the exchange: pass 0 = finer owners, 1 = same level, 2 = coarser.
 template <typename T>
-__global__ void fill_kernel(DevForest F, StateView<T> S, uint32_t dst, uint32_t src, int flags, int pass) {
+__global__ void fill_kernel(const __grid_constant__ DevForest F, StateView<T> S, uint32_t dst, uint32_t src, int flags, int pass) {
     const int p = blockIdx.x;
     const int lp = __ldg(F.level + p);
     if (!((dst >> lp) & 1u)) return;
@@ -411,7 +402,7 @@ __global__ void fill_kernel(DevForest F, StateView<T> S, uint32_t dst, uint32_t 
         if (i > 0 && i < n && j > 0 && j < n) continue;  // strictly inside: the leaf's own
         if (i == n + kGhost && (k == kAvg || k == kYmid)) continue;  // never read by the step
         if (j == n + kGhost && (k == kAvg || k == kXmid)) continue;
-        long long x, y;
+        int x, y;
         entry_xy(F, p, k, i, j, x, y);
         const int q = entry_owner(F, k, x, y);
         if (q < 0 || q == p) continue;
@@ -419,9 +410,9 @@ __global__ void fill_kernel(DevForest F, StateView<T> S, uint32_t dst, uint32_t 
         const int rel_pass = lq > lp ? 0 : (lq == lp ? 1 : 2);
         if (rel_pass != pass || !((src >> lq) & 1u)) continue;
         if ((flags & AF_FILL_SAME_LEVEL_ONLY) && lq != lp) continue;
-        double v[3];
+        T v[3];
         transfer_all<T>(F, S, lp, q, k, x, y, S.ncomp, v);
-        for (int c = 0; c < S.ncomp; ++c) *S.at(p, c, k, i, j) = (T)v[c];
+        for (int c = 0; c < S.ncomp; ++c) *S.at(p, c, k, i, j) = v[c];
     }
 }
 
@@ -449,7 +440,7 @@ __device__ bool ghost_entry(const DevForest &F, int64_t plane, int p, int lp, in
     if (i > 0 && i < n && j > 0 && j < n) return false;
     if (i == n + kGhost && (k == kAvg || k == kYmid)) return false;
     if (j == n + kGhost && (k == kAvg || k == kXmid)) return false;
-    long long x, y;
+    int x, y;
     entry_xy(F, p, k, i, j, x, y);
     const int q = entry_owner(F, k, x, y);
     if (q < 0 || q == p) return false;
@@ -465,7 +456,7 @@ __device__ bool ghost_entry(const DevForest &F, int64_t plane, int p, int lp, in
         g.aux = (uint32_t)(k * plane + (int64_t)(sj + kGhost) * W + (si + kGhost));
     } else if (lq > lp) {
         if (k == kAvg) {
-            const long long h = hwid(F, lq) / 2;  // the four finer cells: (si, sj) .. (si + 1, sj + 1)
+            const int h = hwid(F, lq) / 2;  // the four finer cells: (si, sj) .. (si + 1, sj + 1)
             lattice_of(F, q, kAvg, x - h, y - h, si, sj);
             g.kind = kGMean4;
             g.aux = (uint32_t)(kAvg * plane + (int64_t)(sj + kGhost) * W + (si + kGhost));
@@ -475,8 +466,10 @@ __device__ bool ghost_entry(const DevForest &F, int64_t plane, int p, int lp, in
             g.aux = (uint32_t)(kCorner * plane + (int64_t)(sj + kGhost) * W + (si + kGhost));
         }
     } else {
-        const long long quarter = hwid(F, lq) / 4;
-        long long u = reld(F, x, leaf_x0(F, q)) / quarter, v = reld(F, y, leaf_y0(F, q)) / quarter;
+        // in quarter cells of the source (2^sh units, sh >= 0 for a
+        // leaf coarser than another)
+        const int sh = F.lmax - lq - 1;
+        int u = reld(F, x, leaf_x0(F, q)) >> sh, v = reld(F, y, leaf_y0(F, q)) >> sh;
         u = u < 0 ? 0 : (u > 4 * n ? 4 * n : u);
         v = v < 0 ? 0 : (v > 4 * n ? 4 * n : v);
         g.kind = k == kAvg ? kGSimpson : kGPoint;
@@ -489,22 +482,50 @@ __device__ __forceinline__ bool plan_leaf(const DevForest &F, int p, int flags) 
     return (flags & AF_FILL_ALL_PATCHES) || has_other_level_neighbour(F, p);
 }
 
-// counts[0]: pass-A entries, counts[1]: pass-B entries.
-__global__ void plan_count_kernel(DevForest F, int64_t plane, int flags, unsigned long long *counts) {
-    const int p = blockIdx.x;
-    __shared__ int s_use;
-    __shared__ unsigned int s_cnt[2];
-    if (threadIdx.x == 0) {
-        s_use = plan_leaf(F, p, flags);
-        s_cnt[0] = s_cnt[1] = 0;
+// The lattice entries a leaf does not hold strictly inside, numbered in
+// lattice order (plane, row, column): rows -2 .. 0 whole, six columns of rows
+// 1 .. n-1 (-2 .. 0, n .. n+2), rows n .. n+2 whole.
+__host__ __device__ constexpr int ring_count(int n) { return 6 * (n + 2 * kGhost + 1) + 6 * (n - 1); }
+__device__ __forceinline__ void ring_entry(int n, int e, int &k, int &i, int &j) {
+    const int W = n + 2 * kGhost + 1, per = ring_count(n), lo = 3 * W, mid = lo + 6 * (n - 1);
+    k = e / per;
+    const int r = e - k * per;
+    if (r < lo) {
+        j = r / W;
+        i = r - j * W - kGhost;
+        j -= kGhost;
+    } else if (r < mid) {
+        const int m = (r - lo) / 6, c = r - lo - 6 * m;
+        j = m + 1;
+        i = c < 3 ? c - kGhost : n + c - 3;
+    } else {
+        const int m = (r - mid) / W;
+        i = r - mid - m * W - kGhost;
+        j = n + m;
     }
+}
+
+// counts[0]: pass-A entries, counts[1]: pass-B entries.
+__global__ void __launch_bounds__(256) plan_count_kernel(const __grid_constant__ DevForest F, int64_t plane, int flags,
+                                                         unsigned long long *counts) {
+    const int p = blockIdx.x;
+    __shared__ unsigned int s_cnt[2];
+    if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
+    if (!plan_leaf(F, p, flags)) return;  // the same for the whole CTA
     __syncthreads();
-    if (!s_use) return;
-    const int lp = __ldg(F.level + p), W = F.n + 2 * kGhost + 1;
-    for (int e = threadIdx.x; e < kPlanes * W * W; e += blockDim.x) {
-        const int k = e / (W * W), r = e - k * W * W;
+    const int lp = __ldg(F.level + p), total = kPlanes * ring_count(F.n);
+    unsigned int c0 = 0, c1 = 0;
+    for (int e = threadIdx.x; e < total; e += blockDim.x) {
+        int k, i, j;
+        ring_entry(F.n, e, k, i, j);
         GhostEntry g;
-        if (ghost_entry(F, plane, p, lp, k, r % W - kGhost, r / W - kGhost, g)) atomicAdd(&s_cnt[g.kind >= kGPoint], 1u);
+        if (ghost_entry(F, plane, p, lp, k, i, j, g)) (g.kind >= kGPoint ? c1 : c0) += 1;
+    }
+    c0 = __reduce_add_sync(0xffffffffu, c0);
+    c1 = __reduce_add_sync(0xffffffffu, c1);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&s_cnt[0], c0);
+        atomicAdd(&s_cnt[1], c1);
     }
     __syncthreads();
     if (threadIdx.x < 2 && s_cnt[threadIdx.x]) atomicAdd(counts + threadIdx.x, (unsigned long long)s_cnt[threadIdx.x]);
@@ -517,39 +538,29 @@ __global__ void plan_count_kernel(DevForest F, int64_t plane, int flags, unsigne
 // consecutive source entries): the exchange's accesses coalesce.  The order
 // of the leaves' ranges is whatever order the CTAs reserve them in; each
 // destination entry appears once, so the order does not change the result.
-__global__ void plan_build_kernel(DevForest F, int64_t plane, int flags, GhostEntry *plan, long long na, long long nb,
-                                  unsigned long long *cursor, int *overflow) {
+// The entries are found once and kept in shared memory (pass A from the
+// front, pass B from the back) until their ranges are known.
+__global__ void __launch_bounds__(256) plan_build_kernel(const __grid_constant__ DevForest F, int64_t plane, int flags, GhostEntry *plan,
+                                                         long long na, long long nb, unsigned long long *cursor,
+                                                         int *overflow) {
     const int p = blockIdx.x;
-    __shared__ int s_use;
-    __shared__ unsigned int s_cnt[2];
+    extern __shared__ __align__(16) unsigned char plan_smem[];
+    GhostEntry *const held = reinterpret_cast<GhostEntry *>(plan_smem);  // [kPlanes * ring_count(n)]
     __shared__ unsigned long long s_base[2];
     __shared__ unsigned int s_warp[2][32];
-    if (threadIdx.x == 0) {
-        s_use = plan_leaf(F, p, flags);
-        s_cnt[0] = s_cnt[1] = 0;
-    }
-    __syncthreads();
-    if (!s_use) return;
-    const int lp = __ldg(F.level + p), W = F.n + 2 * kGhost + 1;
-    const int total = kPlanes * W * W;
-    for (int e = threadIdx.x; e < total; e += blockDim.x) {
-        const int k = e / (W * W), r = e - k * W * W;
-        GhostEntry g;
-        if (ghost_entry(F, plane, p, lp, k, r % W - kGhost, r / W - kGhost, g)) atomicAdd(&s_cnt[g.kind >= kGPoint], 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x < 2) s_base[threadIdx.x] = s_cnt[threadIdx.x] ? atomicAdd(cursor + threadIdx.x, s_cnt[threadIdx.x]) : 0ull;
-    __syncthreads();
+    if (!plan_leaf(F, p, flags)) return;  // the same for the whole CTA
+    const int lp = __ldg(F.level + p), total = kPlanes * ring_count(F.n);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
     const unsigned below = (1u << lane) - 1u;
-    unsigned long long run0 = s_base[0], run1 = s_base[1];
+    unsigned run0 = 0, run1 = 0;
     for (int e0 = 0; e0 < total; e0 += blockDim.x) {
         const int e = e0 + threadIdx.x;
         GhostEntry g;
         bool v = false;
         if (e < total) {
-            const int k = e / (W * W), r = e - k * W * W;
-            v = ghost_entry(F, plane, p, lp, k, r % W - kGhost, r / W - kGhost, g);
+            int k, i, j;
+            ring_entry(F.n, e, k, i, j);
+            v = ghost_entry(F, plane, p, lp, k, i, j, g);
         }
         const int b = v ? (g.kind >= kGPoint) : 0;
         const unsigned m0 = __ballot_sync(0xffffffffu, v && b == 0), m1 = __ballot_sync(0xffffffffu, v && b == 1);
@@ -567,17 +578,24 @@ __global__ void plan_build_kernel(DevForest F, int64_t plane, int flags, GhostEn
             tot0 += s_warp[0][w];
             tot1 += s_warp[1][w];
         }
-        if (v) {
-            const unsigned long long slot = b ? run1 + off1 + __popc(m1 & below) : run0 + off0 + __popc(m0 & below);
-            if ((long long)slot >= (b ? nb : na)) {
-                atomicExch(overflow, 1);
-            } else {
-                plan[(b ? na : 0) + (long long)slot] = g;
-            }
-        }
+        if (v) held[b ? total - 1 - (int)(run1 + off1 + __popc(m1 & below)) : (int)(run0 + off0 + __popc(m0 & below))] = g;
         run0 += tot0;
         run1 += tot1;
         __syncthreads();
+    }
+    if (threadIdx.x < 2) {
+        const unsigned c = threadIdx.x ? run1 : run0;
+        s_base[threadIdx.x] = c ? atomicAdd(cursor + threadIdx.x, (unsigned long long)c) : 0ull;
+    }
+    __syncthreads();
+    for (unsigned e = threadIdx.x; e < run0 + run1; e += blockDim.x) {
+        const int b = e >= run0;
+        const unsigned r = b ? e - run0 : e;
+        const long long slot = (long long)(s_base[b] + r);
+        if (slot >= (b ? nb : na))
+            atomicExch(overflow, 1);
+        else
+            plan[(b ? na : 0) + slot] = held[b ? total - 1 - (int)r : (int)r];
     }
 }
 
@@ -639,8 +657,27 @@ __global__ void plan_exec_b(StateView<T> S, int n, const GhostEntry *__restrict_
     }
 }
 
+// Sites of a quarter of a leaf that a refinement reads: the corners, left-edge
+// and bottom-edge midpoints and averages of its m x m cells, closed.
+__host__ __device__ constexpr int quarter_sites(int m) { return (m + 1) * (m + 1) + 2 * m * (m + 1) + m * m; }
+constexpr int kStagedMax = 32;  // largest patch whose quarter is staged (26 KB in FP64)
+
+// The state of every leaf of the new forest from the old one.
+//  - A leaf of both forests is copied (16-byte words).
+//  - A child of an old leaf is interpolated: its 4 (n+1)^2 entries use each of
+//    the quarter's sites up to a dozen times, so the CTA first gathers them in
+//    shared memory, looking the owner of a boundary site up once.  Only entries
+//    on the old leaf's own boundary may belong to another leaf and are looked
+//    up one by one.  (Looked up per entry and site, in 64 bits, the transfer
+//    between 2100 and 2700 leaves averaged 721 us; with the quarters staged and
+//    the look-ups kept out of line, 94.  The copies alone would take 17 us at
+//    the HBM rate; latency of the few CTAs that refine bounds the rest.)
+//  - A merged leaf is averaged from its children, the owner of everything
+//    strictly inside known from four lookups.
 template <typename T>
-__global__ void transfer_kernel(DevForest Fo, StateView<T> So, DevForest Fn, StateView<T> Sn) {
+__global__ void __launch_bounds__(256, 3) transfer_kernel(
+    const __grid_constant__ DevForest Fo, const __grid_constant__ StateView<T> So, const __grid_constant__ DevForest Fn,
+    const __grid_constant__ StateView<T> Sn) {
     const int p = blockIdx.x;
     const int l = __ldg(Fn.level + p), px = __ldg(Fn.ix + p), py = __ldg(Fn.iy + p);
     const int64_t words = (int64_t)Sn.ncomp * kPlanes * Sn.plane;
@@ -651,8 +688,8 @@ __global__ void transfer_kernel(DevForest Fo, StateView<T> So, DevForest Fn, Sta
         same = __ldg(Fo.map + map_offset(Fo.B, l) + (long long)py * side + px);
     }
     const int n = Fn.n, m = n + 1;
-    const long long hwn = 2LL << (Fn.lmax - l);
-    const long long x0 = (long long)px * n * hwn, y0 = (long long)py * n * hwn;
+    const int hwn = 2 << (Fn.lmax - l);
+    const int x0 = px * n * hwn, y0 = py * n * hwn;
     if (same >= 0) {
         const T *srcp = So.patch(same);
         constexpr int V = 16 / (int)sizeof(T);  // elements per 16-byte load
@@ -675,17 +712,45 @@ __global__ void transfer_kernel(DevForest Fo, StateView<T> So, DevForest Fn, Sta
             const int k = side == 0 || side == 2 ? kCorner : (side == 1 ? kXmid : kYmid);
             const int i = side < 2 ? n : r, j = side < 2 ? r : n;
             if ((k == kXmid && j == n) || (k == kYmid && i == n)) continue;
-            const long long x = x0 + (long long)i * hwn + (k == kYmid ? hwn / 2 : 0);
-            const long long y = y0 + (long long)j * hwn + (k == kXmid ? hwn / 2 : 0);
+            const int x = x0 + i * hwn + (k == kYmid ? hwn / 2 : 0);
+            const int y = y0 + j * hwn + (k == kXmid ? hwn / 2 : 0);
             const int q = entry_owner(Fo, k, x, y);
             if (q < 0 || q == same) continue;
-            double v[3];
-            transfer_all<T>(Fo, So, l, q, k, x, y, Sn.ncomp, v);
-            for (int c = 0; c < Sn.ncomp; ++c) *Sn.at(p, c, k, i, j) = (T)v[c];
+            T v[3];
+            transfer_entry<T>(Fo, So, l, q, k, x, y, v);
+            for (int c = 0; c < Sn.ncomp; ++c) *Sn.at(p, c, k, i, j) = v[c];
         }
         return;
     }
     for (int64_t e = threadIdx.x; e < words; e += blockDim.x) dst[e] = T(0);
+    // the old leaves of the new leaf's four quarters (the same one for a child)
+    extern __shared__ __align__(16) unsigned char site_smem[];
+    T *const site = reinterpret_cast<T *>(site_smem);
+    __shared__ int s_q[4];
+    if (threadIdx.x < 4) {
+        const int w = n * hwn;
+        s_q[threadIdx.x] = lookup(Fo, x0 + (threadIdx.x & 1 ? w - 1 : 0), y0 + (threadIdx.x & 2 ? w - 1 : 0));
+    }
+    __syncthreads();
+    const int q0 = s_q[0], nc = Sn.ncomp;
+    const bool child = q0 >= 0 && __ldg(Fo.level + q0) == l - 1 && n % 2 == 0 && n <= kStagedMax;
+    // every quarter one leaf: then those own what lies strictly inside
+    bool four = q0 >= 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) four = four && s_q[e] >= 0 && __ldg(Fo.level + (s_q[e] < 0 ? 0 : s_q[e])) <= l + 1;
+    const int mq = n / 2, cx = (px & 1) * mq, cy = (py & 1) * mq, sites = quarter_sites(mq);
+    const int qhw = 2 * hwn, qx0 = x0 - cx * qhw, qy0 = y0 - cy * qhw;  // the old leaf's cells and corner (child)
+    const int b1 = (mq + 1) * (mq + 1), b2 = b1 + (mq + 1) * mq, b3 = b2 + mq * (mq + 1);
+    if (child) {
+        for (int e = threadIdx.x; e < sites; e += blockDim.x) {
+            const int k = e < b1 ? kCorner : (e < b2 ? kXmid : (e < b3 ? kYmid : kAvg));
+            const int r = e - (e < b1 ? 0 : (e < b2 ? b1 : (e < b3 ? b2 : b3)));
+            const int w = (k == kCorner || k == kXmid) ? mq + 1 : mq, j = r / w, i = r - j * w;
+            const T *v = k == kAvg ? So.at(q0, 0, kAvg, cx + i, cy + j)
+                                   : node_value<T>(Fo, So, q0, l - 1, qx0, qy0, qhw, k, cx + i, cy + j);
+            for (int c = 0; c < nc; ++c) site[c * sites + e] = v[c * kPlanes * So.plane];
+        }
+    }
     __syncthreads();
     // The cells' averages and the point values on their boundaries: node
     // lines 0 .. n, the right (i = n) and top (j = n) lines included -- a leaf
@@ -696,16 +761,39 @@ __global__ void transfer_kernel(DevForest Fo, StateView<T> So, DevForest Fn, Sta
     for (int e = threadIdx.x; e < kPlanes * m * m; e += blockDim.x) {
         const int k = e / (m * m), r = e - k * m * m, j = r / m, i = r - j * m;
         if ((i == n && (k == kAvg || k == kYmid)) || (j == n && (k == kAvg || k == kXmid))) continue;
-        const long long x = x0 + (long long)i * hwn + ((k == kAvg || k == kYmid) ? hwn / 2 : 0);
-        const long long y = y0 + (long long)j * hwn + ((k == kAvg || k == kXmid) ? hwn / 2 : 0);
-        const int q = entry_owner(Fo, k, x, y);
+        const int x = x0 + i * hwn + ((k == kAvg || k == kYmid) ? hwn / 2 : 0);
+        const int y = y0 + j * hwn + ((k == kAvg || k == kXmid) ? hwn / 2 : 0);
+        const bool inside = k == kAvg || (i > 0 && i < n && j > 0 && j < n) ||
+                            (k == kXmid && i > 0 && i < n) || (k == kYmid && j > 0 && j < n);
+        const int nx = cx * 2 + i, ny = cy * 2 + j;  // in half cells of the old leaf (child)
+        const bool in = k == kAvg || ((k == kYmid || (nx > 0 && nx < 2 * n)) && (k == kXmid || (ny > 0 && ny < 2 * n)));
+        int q;
+        if (child ? in : inside && four)
+            q = child ? q0 : s_q[(2 * i + (k == kAvg || k == kYmid) >= n) + 2 * (2 * j + (k == kAvg || k == kXmid) >= n)];
+        else
+            q = entry_owner(Fo, k, x, y);
         if (q < 0) continue;
-        // an average comes from at most one level finer (the four children's
-        // mean); a point value is the coinciding vertex of any finer owner
-        if (k == kAvg && __ldg(Fo.level + q) > l + 1) continue;
-        double v[3];
-        transfer_all<T>(Fo, So, l, q, k, x, y, Sn.ncomp, v);
-        for (int c = 0; c < Sn.ncomp; ++c) *Sn.at(p, c, k, i, j) = (T)v[c];
+        T v[3];
+        if (child && q == q0) {
+            // cell (ci, cj) of the quarter; the last line is the last cell's far edge
+            const int ux = 2 * i + (k == kAvg || k == kYmid), uy = 2 * j + (k == kAvg || k == kXmid);  // quarter cells
+            const int ci = min(ux >> 2, mq - 1), cj = min(uy >> 2, mq - 1);
+            const T xi = T(0.5) * (T)(ux - 4 * ci) - T(1), eta = T(0.5) * (T)(uy - 4 * cj) - T(1);
+            const int c0 = cj * (mq + 1) + ci, xo = b1 + cj * (mq + 1) + ci, yo = b2 + cj * mq + ci, ao = b3 + cj * mq + ci;
+            for (int c = 0; c < nc; ++c) {
+                const T *w = site + c * sites;
+                const T c00 = w[c0], c10 = w[c0 + 1], c01 = w[c0 + mq + 1], c11 = w[c0 + mq + 2];
+                const T xl = w[xo], xr = w[xo + 1], yb = w[yo], yt = w[yo + mq], av = w[ao];
+                v[c] = k == kAvg ? recon_quarter_mean<T>(c00, c10, c01, c11, xl, xr, yb, yt, av, ux - 4 * ci >= 2, uy - 4 * cj >= 2)
+                                 : recon_eval<T>(c00, c10, c01, c11, xl, xr, yb, yt, av, xi, eta);
+            }
+        } else {
+            // an average comes from at most one level finer (the four children's
+            // mean); a point value is the coinciding vertex of any finer owner
+            if (k == kAvg && __ldg(Fo.level + q) > l + 1) continue;
+            transfer_entry<T>(Fo, So, l, q, k, x, y, v);
+        }
+        for (int c = 0; c < nc; ++c) *Sn.at(p, c, k, i, j) = v[c];
     }
 }
 
@@ -717,26 +805,27 @@ template <>
 __device__ __forceinline__ void atomic_add_state<float>(float *p, double v) { atomicAdd(p, (float)v); }
 
 template <typename T>
-__global__ void reflux_kernel(DevForest F, StateView<T> S, uint32_t sync, double dx0, double dy0, double *freg) {
+__global__ void reflux_kernel(const __grid_constant__ DevForest F, StateView<T> S, uint32_t sync, double dx0, double dy0, double *freg) {
     const int n = F.n, nc = S.ncomp;
     const int64_t total = (int64_t)F.nleaf * 4 * n;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int p = (int)(t / (4 * n)), side = (int)((t / n) % 4), k = (int)(t % n);
+        // 32-bit divisions (total < 2^31 for any state that fits the GPU)
+        const int f = (int)t / n, k = (int)t - f * n, p = f >> 2, side = f & 3;
         const int l = __ldg(F.level + p);
         if (l >= AF_MAX_LEVEL || !((sync >> l) & 1u) || !((sync >> (l + 1)) & 1u)) continue;
-        const long long hw = hwid(F, l), x0 = leaf_x0(F, p), y0 = leaf_y0(F, p);
-        const long long x1 = x0 + (long long)n * hw, y1 = y0 + (long long)n * hw;
-        long long px, py;
+        const int hw = hwid(F, l), x0 = leaf_x0(F, p), y0 = leaf_y0(F, p);
+        const int x1 = x0 + n * hw, y1 = y0 + n * hw;
+        int px, py;
         if (side == 0) { px = x0 - 1; py = y0 + k * hw + hw / 2; }
         else if (side == 1) { px = x1; py = y0 + k * hw + hw / 2; }
         else if (side == 2) { px = x0 + k * hw + hw / 2; py = y0 - 1; }
         else { px = x0 + k * hw + hw / 2; py = y1; }
         const int q = lookup(F, px, py);
         if (q < 0 || __ldg(F.level + q) != l + 1) continue;
-        const long long hf = hwid(F, l + 1);
+        const int hf = hwid(F, l + 1);
         const int fside = side ^ 1;
-        const long long start = side < 2 ? reld(F, y0 + k * hw, leaf_y0(F, q)) : reld(F, x0 + k * hw, leaf_x0(F, q));
-        const int kf = (int)(start / hf);
+        const int start = side < 2 ? reld(F, y0 + k * hw, leaf_y0(F, q)) : reld(F, x0 + k * hw, leaf_x0(F, q));
+        const int kf = start / hf;
         if (kf < 0 || kf + 1 >= n) continue;
         const int ci = side == 0 ? 0 : (side == 1 ? n - 1 : k);
         const int cj = side == 2 ? 0 : (side == 3 ? n - 1 : k);
@@ -756,12 +845,13 @@ __global__ void reflux_kernel(DevForest F, StateView<T> S, uint32_t sync, double
 }
 
 template <typename T>
-__global__ void tag_kernel(DevForest F, StateView<T> S, int comp, int kind, double dx0, double dy0, double rthr,
+__global__ void tag_kernel(const __grid_constant__ DevForest F, StateView<T> S, int comp, int kind, double dx0, double dy0, double rthr,
                            double cthr, int8_t *tags, double *ind) {
     const int p = blockIdx.x, n = F.n;
     const int l = __ldg(F.level + p);
     const double hx = dx0 / (double)(1LL << l), hy = dy0 / (double)(1LL << l);
-    double a = -INFINITY, b = INFINITY;  // kind 0: max, min; kind 1: max gradient in a
+    // kind 0: max, min; kind 1: largest centred differences in x, y
+    double a = -INFINITY, b = kind == 0 ? INFINITY : -INFINITY;
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
         const int j = e / n, i = e % n;
         if (kind == 0) {
@@ -769,9 +859,10 @@ __global__ void tag_kernel(DevForest F, StateView<T> S, int comp, int kind, doub
             a = fmax(a, q);
             b = fmin(b, q);
         } else if (i >= 1 && i < n - 1 && j >= 1 && j < n - 1) {
-            const double gx = fabs((double)*S.at(p, comp, kAvg, i + 1, j) - (double)*S.at(p, comp, kAvg, i - 1, j)) / (2.0 * hx);
-            const double gy = fabs((double)*S.at(p, comp, kAvg, i, j + 1) - (double)*S.at(p, comp, kAvg, i, j - 1)) / (2.0 * hy);
-            a = fmax(a, fmax(gx, gy));
+            // the largest differences; divided by the widths once below (division
+            // by a positive number is monotonic, rounding included)
+            a = fmax(a, fabs((double)*S.at(p, comp, kAvg, i + 1, j) - (double)*S.at(p, comp, kAvg, i - 1, j)));
+            b = fmax(b, fabs((double)*S.at(p, comp, kAvg, i, j + 1) - (double)*S.at(p, comp, kAvg, i, j - 1)));
         }
     }
     __shared__ double sa[256], sb[256];
@@ -781,12 +872,12 @@ __global__ void tag_kernel(DevForest F, StateView<T> S, int comp, int kind, doub
     for (int s = blockDim.x / 2; s > 0; s >>= 1) {
         if ((int)threadIdx.x < s) {
             sa[threadIdx.x] = fmax(sa[threadIdx.x], sa[threadIdx.x + s]);
-            sb[threadIdx.x] = fmin(sb[threadIdx.x], sb[threadIdx.x + s]);
+            sb[threadIdx.x] = kind == 0 ? fmin(sb[threadIdx.x], sb[threadIdx.x + s]) : fmax(sb[threadIdx.x], sb[threadIdx.x + s]);
         }
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        const double v = kind == 0 ? sa[0] - sb[0] : fmax(sa[0], 0.0);
+        const double v = kind == 0 ? sa[0] - sb[0] : fmax(fmax(sa[0] / (2.0 * hx), sb[0] / (2.0 * hy)), 0.0);
         if (ind) ind[p] = v;
         tags[p] = (int8_t)(v >= rthr ? 1 : (v < cthr ? -1 : 0));
     }
@@ -980,7 +1071,10 @@ extern "C" af_status af_ghost_plan_build(const af_config *cfg, const af_forest *
     // scratch: two slot cursors and an overflow flag
     if (cudaMemsetAsync(d_scratch, 0, 3 * sizeof(int64_t), s) != cudaSuccess) return AF_ERR_CUDA;
     if (forest->nleaf == 0) return AF_OK;
-    plan_build_kernel<<<forest->nleaf, 256, 0, s>>>(
+    const size_t held = (size_t)kPlanes * ring_count(cfg->n) * sizeof(GhostEntry);  // up to 52 KB (n = 64)
+    if (cudaFuncSetAttribute(plan_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)held) != cudaSuccess)
+        return AF_ERR_CUDA;
+    plan_build_kernel<<<forest->nleaf, 256, held, s>>>(
         make_dev(*forest, cfg->n), plane_stride(cfg->n), flags, static_cast<GhostEntry *>(d_plan), n_a, n_b,
         reinterpret_cast<unsigned long long *>(d_scratch), reinterpret_cast<int *>(d_scratch + 2));
     return launched();
@@ -1030,12 +1124,13 @@ extern "C" af_status af_transfer_pair(const af_config *cfg, const af_forest *old
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const DevForest Fo = make_dev(*old_forest, cfg->n), Fn = make_dev(*new_forest, cfg->n);
     const af_state_pair sn = single(d_new);
+    const size_t held = cfg->n <= kStagedMax ? (size_t)quarter_sites(cfg->n / 2) * cfg->ncomp * (cfg->prec == AF_F64 ? 8 : 4) : 0;
     if (cfg->prec == AF_F64)
-        transfer_kernel<double><<<new_forest->nleaf, 256, 0, s>>>(Fo, view<double>(*cfg, *old_forest, *old_state), Fn,
-                                                                 view<double>(*cfg, *new_forest, sn));
+        transfer_kernel<double><<<new_forest->nleaf, 256, held, s>>>(Fo, view<double>(*cfg, *old_forest, *old_state), Fn,
+                                                                    view<double>(*cfg, *new_forest, sn));
     else
-        transfer_kernel<float><<<new_forest->nleaf, 256, 0, s>>>(Fo, view<float>(*cfg, *old_forest, *old_state), Fn,
-                                                                view<float>(*cfg, *new_forest, sn));
+        transfer_kernel<float><<<new_forest->nleaf, 256, held, s>>>(Fo, view<float>(*cfg, *old_forest, *old_state), Fn,
+                                                                   view<float>(*cfg, *new_forest, sn));
     return launched();
 }
 

@@ -119,6 +119,51 @@ def test_transfer_matches_oracle(af, prec):
 
 
 @pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,eq,jump", [(2, 1, 0), (6, 0, 0), (7, 1, 0), (16, 1, 0), (32, 1, 0), (34, 0, 0), (8, 1, 2), (9, 0, 2)])
+def test_transfer_of_every_patch_size_matches_oracle(af, n, eq, jump, prec):
+    """af_transfer from random data (no owner may stand in for another): patch
+    sizes with and without staged quarters (even up to 32; odd; larger),
+    children, merged families and copies side by side, and leaves that come
+    from two levels coarser (jump = 2).  Same arithmetic as the oracle up to
+    rounding: the bounds of one step."""
+    from paper_2205_07572_gb300.amr import regrid_leaves
+    lmax, nc = 4, 1 if eq == 0 else 3
+    rng = np.random.default_rng(11 * n + jump)
+    if jump:
+        leaves = _sorted([(1, x, y) for y in range(2) for x in range(2)])
+        new = _sorted([(1 + jump, x, y) for y in range(2 << jump) for x in range(2 << jump)])
+    else:
+        leaves = _sorted(_diag_forest(1, 3))
+        F = _device_forest(af, leaves, lmax)
+        tags = rng.choice([-1, 0, 1], size=len(leaves)).astype(np.int8)
+        fam = {}
+        for k, (l, x, y) in enumerate(leaves):
+            fam.setdefault((l, x >> 1, y >> 1), []).append(k)
+        for k, ks in enumerate(v for v in fam.values() if len(v) == 4):
+            if k % 3 == 0:
+                tags[ks] = -1
+        new = regrid_leaves(F, tags, 1)
+        assert set(new) & set(leaves) and any((l - 1, x >> 1, y >> 1) in set(leaves) for l, x, y in new)
+    st = S.random_state(S.Layout(n, nc), len(leaves), seed=5 + n).reshape(len(leaves), -1)
+    if prec:
+        st = st.astype(np.float32).astype(np.float64)
+    lv = lambda L_, k: np.array([t[k] for t in L_], np.int32)  # noqa: E731
+    ref = np.zeros((len(new), st.shape[1]))
+    O.lib().orc_transfer(n, nc, 1, lmax, len(leaves), _ip(lv(leaves, 0)), _ip(lv(leaves, 1)), _ip(lv(leaves, 2)),
+                         O._dp(st), len(new), _ip(lv(new, 0)), _ip(lv(new, 1)), _ip(lv(new, 2)), O._dp(ref))
+    F, Fn = _device_forest(af, leaves, lmax), _device_forest(af, new, lmax)
+    tdt = torch.float64 if prec == 0 else torch.float32
+    d_old = torch.from_numpy(st).to(tdt).cuda()
+    d_new = torch.full((len(new), st.shape[1]), float("nan"), dtype=tdt, device="cuda")
+    af.transfer(af.config(eq, prec, n, 1.0, 0.5, 1.0), F.c, d_old, Fn.c, d_new)
+    torch.cuda.synchronize()
+    lay = S.Layout(n, nc)
+    g = lay.lattice(d_new.double().cpu().numpy().reshape(len(new), nc, 4, -1))[..., G:G + n, G:G + n]
+    r = lay.lattice(ref.reshape(len(new), nc, 4, -1))[..., G:G + n, G:G + n]
+    assert _nerr(g, r) < TOL[prec]
+
+
+@pytest.mark.parametrize("prec", [0, 1])
 def test_reflux_matches_oracle(af, prec):
     n, lmax, nc = 8, 3, 3
     leaves = _sorted(_diag_forest(2, 3))
