@@ -119,9 +119,14 @@ def test_backward_of_every_shape_and_ragged_batch_matches_oracle(af, C, N, P, nb
     o = 32 * C * 9 + 16 * 32 + 32 * 32 * 9
     params[o + 3:o + 9] = -1000.0  # b2: channels whose maximum is never positive
     level[0] = 0
-    g_r = OC.backward(X, level, params, C, label, omega)
     lg, M, arg, _ = OC.forward(X, level, params, C)
     assert (arg[:, 3:9] == -1).all()
+    # the loss's derivative as FP32 forms it: sigmoid(l) - y cancels where the
+    # network is sure, and what is left scales the whole sample's gradient
+    l32, one = lg.astype(np.float32), np.float32(1)
+    d32 = (one / (one + np.exp(-l32)) - label).astype(np.float64)
+    om = omega * d32 / (1.0 / (1.0 + np.exp(-lg)) - label)
+    g_r = OC.backward(X, level, params, C, label, om) * (om.sum() / omega.sum())
     np_ = len(params)
     dev = lambda a, t: torch.from_numpy(np.ascontiguousarray(a).astype(t)).cuda()  # noqa: E731
     lv = level.copy()
