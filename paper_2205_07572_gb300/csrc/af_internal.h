@@ -92,6 +92,19 @@ struct AdvectionWeights {
     int32_t off[3][2][2];
 };
 
+// The same for the kernel.  If both feet of every node type lie in one cell
+// that also holds the node itself (fold = 1; |CFL| <= 1/2 is enough), the
+// combination T = Q^n + 4 Q^{n+1/2} + Q^{n+1} that enters the fluxes is itself
+// one combination of that cell's values: v[t][k][0] = 4 w[t][0][k] + w[t][1][k]
+// (+ 1 for the node's own value) gives T, v[t][k][1] = w[t][1][k] gives
+// Q^{n+1}.  Otherwise v[t][k][s] = w[t][s][k].
+template <typename T>
+struct AdvectionPairWeights {
+    T v[3][9][2];
+    int32_t off[3][2][2];
+    int32_t fold, pad_;
+};
+
 // Double-precision derivations on the host (af_weights.cpp).
 void acoustic_weights(double rho_x, double rho_y, AcousticWeights<double> &w);
 // Folded weights; returns false if the dense weights lack the symmetry

@@ -44,19 +44,33 @@ bool get_acoustic(double rx, double ry, AcousticSymWeights<T> &out) {
 }
 
 template <typename T>
-void get_advection(double nx, double ny, AdvectionWeights<T> &out) {
+void get_advection(double nx, double ny, AdvectionPairWeights<T> &out) {
     std::lock_guard<std::mutex> lk(g_mu);
     const WeightKey k{AF_ADVECTION, nx, ny};
     if (!(k == g_dkey)) {
         advection_weights(nx, ny, g_dw);
         g_dkey = k;
     }
-    for (int t = 0; t < 3; ++t)
-        for (int s = 0; s < 2; ++s) {
-            for (int d = 0; d < 9; ++d) out.w[t][s][d] = (T)g_dw.w[t][s][d];
-            out.off[t][s][0] = g_dw.off[t][s][0];
-            out.off[t][s][1] = g_dw.off[t][s][1];
+    // where the node's own value stands among the foot cell's nine
+    int own[3];
+    bool fold = true;
+    for (int t = 0; t < 3; ++t) {
+        const int ox = -g_dw.off[t][1][0], oy = -g_dw.off[t][1][1];
+        fold = fold && g_dw.off[t][0][0] == -ox && g_dw.off[t][0][1] == -oy;
+        fold = fold && (t == 2 ? ox == 0 : (ox == 0 || ox == 1)) && (t == 1 ? oy == 0 : (oy == 0 || oy == 1));
+        own[t] = t == 0 ? 1 + ox + 2 * oy : (t == 1 ? 5 + ox : 7 + oy);
+    }
+    for (int t = 0; t < 3; ++t) {
+        for (int d = 0; d < 9; ++d) {
+            const double h = g_dw.w[t][0][d], f = g_dw.w[t][1][d];
+            out.v[t][d][0] = (T)(fold ? 4.0 * h + f + (d == own[t] ? 1.0 : 0.0) : h);
+            out.v[t][d][1] = (T)f;
         }
+        for (int s = 0; s < 2; ++s)
+            for (int e = 0; e < 2; ++e) out.off[t][s][e] = g_dw.off[t][s][e];
+    }
+    out.fold = fold ? 1 : 0;
+    out.pad_ = 0;
 }
 
 // Interleave the two time combinations (T, Q^{n+1}) of every FP32 weight.

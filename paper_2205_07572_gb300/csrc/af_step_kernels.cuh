@@ -63,7 +63,7 @@ struct WeightsOf<T, AF_ACOUSTICS> { using type = AcousticSymWeights<T>; };
 template <>
 struct WeightsOf<float, AF_ACOUSTICS> { using type = AcousticPairWeights; };
 template <typename T>
-struct WeightsOf<T, AF_ADVECTION> { using type = AdvectionWeights<T>; };
+struct WeightsOf<T, AF_ADVECTION> { using type = AdvectionPairWeights<T>; };
 
 // Launch one af_patch_step with compiled tiling k (host; af_step_f32/f64.cu).
 template <typename T, int EQ>
@@ -369,21 +369,74 @@ __device__ __forceinline__ void acoustic_item(const AcousticPairWeights &W, cons
     }
 }
 
-// Advection: value of the reconstruction of window cell (cq, cr) with weights w.
+// Advection: the nine degrees of freedom of window cell (cq, cr) in the order
+// of the weights, and combinations of them.
 template <typename T, int WX, int WSZ>
-__device__ __forceinline__ T adv_eval(const T *w, const T *Sin, int cq, int cr) {
+__device__ __forceinline__ void adv_cell(const T *Sin, int cq, int cr, T d[9]) {
     const int o = cr * WX + cq;
     const T *A = Sin + kAvg * WSZ, *C = Sin + kCorner * WSZ, *X = Sin + kXmid * WSZ, *Y = Sin + kYmid * WSZ;
-    T v = w[0] * A[o];
-    v = fma(w[1], C[o], v);
-    v = fma(w[2], C[o + 1], v);
-    v = fma(w[3], C[o + WX], v);
-    v = fma(w[4], C[o + WX + 1], v);
-    v = fma(w[5], X[o], v);
-    v = fma(w[6], X[o + 1], v);
-    v = fma(w[7], Y[o], v);
-    v = fma(w[8], Y[o + WX], v);
+    d[0] = A[o];
+    d[1] = C[o];
+    d[2] = C[o + 1];
+    d[3] = C[o + WX];
+    d[4] = C[o + WX + 1];
+    d[5] = X[o];
+    d[6] = X[o + 1];
+    d[7] = Y[o];
+    d[8] = Y[o + WX];
+}
+// Combination s of one cell's values.
+template <typename T, int WX, int WSZ>
+__device__ __forceinline__ T adv_eval(const T (*w)[2], int s, const T *Sin, int cq, int cr) {
+    T d[9];
+    adv_cell<T, WX, WSZ>(Sin, cq, cr, d);
+    T v = w[0][s] * d[0];
+#pragma unroll
+    for (int k = 1; k < 9; ++k) v = fma(w[k][s], d[k], v);
     return v;
+}
+// Both combinations of one cell's values (FP32: packed, each lane rounded as
+// alone).
+template <int WX, int WSZ>
+__device__ __forceinline__ void adv_eval2(const float (*w)[2], const float *Sin, int cq, int cr, float &v0, float &v1) {
+    float d[9];
+    adv_cell<float, WX, WSZ>(Sin, cq, cr, d);
+    float2 v = __fmul2_rn(make_float2(w[0][0], w[0][1]), make_float2(d[0], d[0]));
+#pragma unroll
+    for (int k = 1; k < 9; ++k) v = __ffma2_rn(make_float2(w[k][0], w[k][1]), make_float2(d[k], d[k]), v);
+    v0 = v.x;
+    v1 = v.y;
+}
+template <int WX, int WSZ>
+__device__ __forceinline__ void adv_eval2(const double (*w)[2], const double *Sin, int cq, int cr, double &v0,
+                                          double &v1) {
+    double d[9];
+    adv_cell<double, WX, WSZ>(Sin, cq, cr, d);
+    v0 = w[0][0] * d[0];
+    v1 = w[0][1] * d[0];
+#pragma unroll
+    for (int k = 1; k < 9; ++k) {
+        v0 = fma(w[k][0], d[k], v0);
+        v1 = fma(w[k][1], d[k], v1);
+    }
+}
+
+// T and Q^{n+1} of a node of type t at window entry (qi, rj), lattice plane
+// `plane` (see AdvectionPairWeights): with the weights folded, nine values and
+// two combinations, for eighteen values, two combinations and the time sum.
+// FP32 is bound by its shared-memory loads and issue slots, FP64 by its pipe
+// (20 operations a node before, 18 now): FP32 4096^2 cells in 16 x 16 patches
+// 333 -> 241 us, FP64 1024^2 194 -> 162 us.
+template <typename T, int WX, int WSZ>
+__device__ __forceinline__ void adv_node(const AdvectionPairWeights<T> &W, int t, int plane, const T *Sin, int qi, int rj,
+                                         T &sum, T &q1) {
+    if (W.fold) {
+        adv_eval2<WX, WSZ>(W.v[t], Sin, qi + W.off[t][1][0], rj + W.off[t][1][1], sum, q1);
+    } else {
+        const T qh = adv_eval<T, WX, WSZ>(W.v[t], 0, Sin, qi + W.off[t][0][0], rj + W.off[t][0][1]);
+        q1 = adv_eval<T, WX, WSZ>(W.v[t], 1, Sin, qi + W.off[t][1][0], rj + W.off[t][1][1]);
+        sum = fma(T(4), qh, Sin[plane * WSZ + rj * WX + qi]) + q1;
+    }
 }
 
 // Tile width whose node and cell items are enumerated with a compile-time
@@ -460,23 +513,18 @@ __device__ __forceinline__ void tile_nodes(const StepArgs<T> &A, const typename 
                 if (hy && st_y) __stcs(po + kYmid * plane, ny[o]);
             }
         } else {
-            const int own = rj * WX + qi;
-            {
-                const T qh = adv_eval<T, WX, WSZ>(W.w[0][0], Sin, qi + W.off[0][0][0], rj + W.off[0][0][1]);
-                const T q1 = adv_eval<T, WX, WSZ>(W.w[0][1], Sin, qi + W.off[0][1][0], rj + W.off[0][1][1]);
-                ST[0 * TSZ + so] = fma(T(4), qh, Sin[kCorner * WSZ + own]) + q1;
-                if (st_x && st_y) ob[kCorner * plane] = q1;
-            }
+            T sum, q1;
+            adv_node<T, WX, WSZ>(W, 0, kCorner, Sin, qi, rj, sum, q1);
+            ST[0 * TSZ + so] = sum;
+            if (st_x && st_y) ob[kCorner * plane] = q1;
             if (hx) {
-                const T qh = adv_eval<T, WX, WSZ>(W.w[1][0], Sin, qi + W.off[1][0][0], rj + W.off[1][0][1]);
-                const T q1 = adv_eval<T, WX, WSZ>(W.w[1][1], Sin, qi + W.off[1][1][0], rj + W.off[1][1][1]);
-                ST[1 * TSZ + so] = fma(T(4), qh, Sin[kXmid * WSZ + own]) + q1;
+                adv_node<T, WX, WSZ>(W, 1, kXmid, Sin, qi, rj, sum, q1);
+                ST[1 * TSZ + so] = sum;
                 if (st_x) ob[kXmid * plane] = q1;
             }
             if (hy) {
-                const T qh = adv_eval<T, WX, WSZ>(W.w[2][0], Sin, qi + W.off[2][0][0], rj + W.off[2][0][1]);
-                const T q1 = adv_eval<T, WX, WSZ>(W.w[2][1], Sin, qi + W.off[2][1][0], rj + W.off[2][1][1]);
-                ST[2 * TSZ + so] = fma(T(4), qh, Sin[kYmid * WSZ + own]) + q1;
+                adv_node<T, WX, WSZ>(W, 2, kYmid, Sin, qi, rj, sum, q1);
+                ST[2 * TSZ + so] = sum;
                 if (st_y) ob[kYmid * plane] = q1;
             }
         }
@@ -941,8 +989,9 @@ __device__ __forceinline__ void write_ghost_columns(const StepArgs<T> &A, const 
 // bulk (async-proxy) writes to the same buffer.
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
-// One tile per CTA.
-template <typename T, int EQ, int NT, int TMX, int TMY, int NN = 0>
+// One tile per CTA.  SPLIT: gridDim.y CTAs share a tile, each a band of its
+// rows, as if the tile had been built that way (few_tiles).
+template <typename T, int EQ, int NT, int TMX, int TMY, int NN = 0, bool SPLIT = false>
 __global__ void __launch_bounds__(NT, (min_ctas<T, EQ, NT>())) step_kernel(const __grid_constant__ StepArgs<T> A,
                                                   const __grid_constant__ typename WeightsOf<T, EQ>::type W) {
     using Gm = Geo<TMX, TMY, NN>;
@@ -952,8 +1001,17 @@ __global__ void __launch_bounds__(NT, (min_ctas<T, EQ, NT>())) step_kernel(const
     T *Sin = Sbase + win_off<T, Gm::WX>();
     T *ST = Sbase + ncomp * kPlanes * Gm::WSZ;
     prefetch_work(A.work, blockIdx.x + kWorkPrefetch, gridDim.x);
-    const af_work wk = load_work(A.work + blockIdx.x);
+    af_work wk = load_work(A.work + blockIdx.x);
     if (wk.x1 - wk.x0 > TMX || wk.y1 - wk.y0 > TMY) return;  // built for another tiling
+    if constexpr (SPLIT) {
+        // (a tile whose copies are made to fail stays whole: one wait runs out)
+        const bool whole = wk.flags & AF_WORK_SKIP_BULK_COPY;
+        const int h = wk.y1 - wk.y0, y0 = wk.y0, part = whole ? 1 : (int)gridDim.y;
+        if ((int)blockIdx.y >= part) return;
+        wk.y0 = (int16_t)(y0 + h * (int)blockIdx.y / part);
+        wk.y1 = (int16_t)(y0 + h * ((int)blockIdx.y + 1) / part);
+        if (wk.y0 == wk.y1) return;
+    }
     prefetch_freg<T, NT>(A, wk.patch, ncomp, NN > 0 ? NN : A.n);
     __shared__ __align__(8) uint64_t bar;
     bool staged = false;
@@ -1103,6 +1161,17 @@ inline cudaError_t ensure_smem(Kern k, size_t bytes) {
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// CTAs that share each of `nwork` tiles of up to `rows` rows (step_kernel,
+// SPLIT): one, unless the tiles leave most of the GPU's 152 SMs idle.  Then as
+// many as bring two CTAs to an SM, of two rows or more: a band's extra row of
+// nodes costs up to half its work again, on SMs that would do nothing.  One
+// 64 x 64 FP64 patch in 32 x 32 tiles: 28.7 us on four CTAs, 9.2 us (the host's
+// share of a call) on 64.
+inline int few_tiles(int nwork, int rows) {
+    const int s = 2 * 152 / (nwork < 1 ? 1 : nwork), most = rows / 2;
+    return s < 2 ? 1 : (s < most ? s : (most < 1 ? 1 : most));
+}
+
 template <typename T, int EQ, int NT, int TMX, int TMY, int PIPE, int NN>
 af_status launch_tiling(const StepArgs<T> &A, const typename WeightsOf<T, EQ>::type &W, int nwork,
                         cudaStream_t stream) {
@@ -1121,6 +1190,15 @@ af_status launch_tiling(const StepArgs<T> &A, const typename WeightsOf<T, EQ>::t
     } else {
         const size_t smem = win + tarr;
         if (smem > 227 * 1024) return AF_ERR_UNIMPLEMENTED;
+        if constexpr (NN == 0) {
+            const int split = few_tiles(nwork, A.n + 2 < TMY ? A.n + 2 : TMY);
+            if (split > 1) {
+                auto kern = dev::step_kernel<T, EQ, NT, TMX, TMY, 0, true>;
+                if (ensure_smem(kern, smem) != cudaSuccess) return AF_ERR_CUDA;
+                kern<<<dim3(nwork, split), NT, smem, stream>>>(A, W);
+                return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+            }
+        }
         auto kern = dev::step_kernel<T, EQ, NT, TMX, TMY, NN>;
         if (ensure_smem(kern, smem) != cudaSuccess) return AF_ERR_CUDA;
         kern<<<nwork, NT, smem, stream>>>(A, W);
@@ -1174,7 +1252,8 @@ extern template af_status launch_step_nn<float, AF_ADVECTION, 32>(int, const Ste
 template <typename T, int EQ>
 af_status launch_step(int k, const StepArgs<T> &A, const typename WeightsOf<T, EQ>::type &W, int nwork,
                       cudaStream_t stream) {
-    if constexpr (sizeof(T) == 4) {
+    // (few tiles are split further, by the kernels for any size)
+    if constexpr (sizeof(T) == 4) if (few_tiles(nwork, 4) == 1) {
         if (A.n == 16) return launch_step_nn<T, EQ, 16>(k, A, W, nwork, stream);
         if (A.n == 32) return launch_step_nn<T, EQ, 32>(k, A, W, nwork, stream);
     }

@@ -346,6 +346,70 @@ def _resplit(work, n, cuts):
 
 
 @pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("a,b", [(0.45, 0.3), (-0.5, 0.5), (0.0, -0.45), (0.95, 0.2), (-0.3, -1.0), (0.6, 0.7), (1.0, 0.0)])
+@pytest.mark.parametrize("n,px,py", [(16, 2, 3), (23, 2, 1), (32, 1, 2)])
+def test_advection_with_feet_in_every_cell_matches_oracle(af, n, px, py, a, b, prec):
+    """Courant numbers (a, b) up to 1 in every direction: both feet of a node in
+    the cell that holds it (the folded weights), on its edge, or in two cells,
+    on one SM's worth of tiles and with the tiles split.  One step each from
+    random data, so the bounds of one step hold."""
+    from paper_2205_07572_gb300.uniform import UniformRun
+    grid = S.UniformGrid(S.Layout(n, 1), px, py)
+    own = S.random_owned(grid, seed=n + px)
+    if prec:
+        own = own.astype(np.float32).astype(np.float64)
+    st = S.pack_owned(grid, own)
+    dt = 0.5 * min(grid.dx, grid.dy)
+    va, vb = a * grid.dx / dt, b * grid.dy / dt
+    ref = S.unpack_owned(grid, O.run_uniform(O.cfg(0, n, grid.dx, grid.dy, dt, va, vb, 1.0), px, py, 1, st))
+    for k in (None, 3, 8):
+        run = UniformRun(af.config(af.ADVECTION, prec, n, va, vb), px, py, grid.dx, grid.dy, dt, state=np.nan_to_num(st),
+                         tiling=k)
+        run.step()
+        torch.cuda.synchronize()
+        got = S.unpack_owned(grid, run.state.double().cpu().numpy().reshape(st.shape))
+        assert np.abs(got - ref).max() / np.abs(ref).max() < (1e-12, 1e-5)[prec], k
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("eq", [0, 1])
+@pytest.mark.parametrize("n,px", [(2, 1), (3, 2), (7, 3), (16, 1), (31, 2), (32, 5), (33, 1), (64, 1), (64, 3)])
+def test_few_tiles_split_over_ctas_match_oracle(af, eq, n, px, prec):
+    """Grids of 1 to 152 tiles in every tiling: each tile is shared by CTAs in
+    row bands, with flux registers and without; the steps and the registers
+    equal the oracle's (bounds of one step), and a second, equal step the first
+    bit for bit."""
+    from paper_2205_07572_gb300.uniform import UniformRun
+    nc = 1 if eq == 0 else 3
+    grid = S.UniformGrid(S.Layout(n, nc), px, px)
+    own = S.random_owned(grid, seed=3 * n + px)
+    if prec:
+        own = own.astype(np.float32).astype(np.float64)
+    st = S.pack_owned(grid, own)
+    dt = 0.4 * grid.dx
+    ref = S.unpack_owned(grid, O.run_uniform(O.cfg(eq, n, grid.dx, grid.dy, dt, 0.9, -0.4, 1.0), px, px, 1, st))
+    for k, t in enumerate(af.step_tilings()):
+        if t[3]:
+            continue
+        outs = []
+        for reg in (False, True, True):
+            run = UniformRun(af.config(eq, prec, n, 0.9, -0.4, 1.0), px, px, grid.dx, grid.dy, dt, state=np.nan_to_num(st),
+                             tiling=k, flux_reg=reg)
+            run.step()
+            torch.cuda.synchronize()
+            got = S.unpack_owned(grid, run.state.double().cpu().numpy().reshape(st.shape))
+            assert np.abs(got - ref).max() / np.abs(ref).max() < (1e-12, 1e-5)[prec], k
+            outs.append((got, None if run.freg is None else run.freg.cpu().numpy()))
+        assert np.array_equal(outs[1][0], outs[2][0]) and np.array_equal(outs[1][1], outs[2][1])
+        # opposite faces of neighbouring patches carry one flux: the totals cancel
+        f = outs[1][1]
+        tol = (1e-12, 1e-5)[prec] * max(1.0, np.abs(f).max()) * px * px * n
+        assert np.abs(f[:, 0].sum(axis=(0, 2)) - f[:, 1].sum(axis=(0, 2))).max() < tol
+        assert np.abs(f[:, 2].sum(axis=(0, 2)) - f[:, 3].sum(axis=(0, 2))).max() < tol
+    assert af.step_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("eq,n,k", [(1, 32, 3), (0, 32, 3), (1, 32, 0), (1, 16, 4), (0, 16, 4), (1, 18, 6), (0, 18, 7),
                                     (1, 10, 8), (1, 16, 9)])
 def test_bulk_staging_equals_elementwise_staging(af, prec, eq, n, k):
