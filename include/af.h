@@ -233,6 +233,33 @@ af_status af_patch_step_pair(const af_config *cfg, int32_t tiling, int32_t nwork
 af_status af_pack_owned(const af_config *cfg, int32_t npatch, const void *d_state, void *d_owned, void *stream);
 af_status af_unpack_owned(const af_config *cfg, int32_t npatch, const void *d_owned, void *d_state, void *stream);
 
+/* One step of npatch patches whose state is kept in HOST memory and updated in
+ * place, as `nband` bands of consecutive patches: band k (patches
+ * [p0, p1), work items d_work[0 .. nwork) of tiling `tiling`, which read the
+ * patches of this and the two neighbouring bands only, cyclically) is copied
+ * to the device on stream s_in, advanced on s_cmp once it and its neighbouring
+ * bands are there, and copied back on s_out, so that both copy directions and
+ * the step overlap.  Bands are advanced in the order 1, 2, .., nband - 1, 0.
+ * Everything is enqueued behind `stream` and joined back into it.
+ *
+ * owned != 0: h_state holds the compact owned layout (af_pack_owned), and
+ *   d_up, d_down are device buffers of its size; each band is unpacked from
+ *   d_up into d_a and packed from d_b into d_down;
+ * owned == 0: h_state holds the state layout; d_up, d_down are unused.
+ * d_a, d_b, dt0, dx0, dy0, d_flux_reg as for af_patch_step (d_in, d_out).
+ * h_state should be pinned; it and all buffers must stay valid until `stream`
+ * has reached this point.  AF_ERR_ARG on NULL pointers, nband < 1 or a band
+ * with p0 < 0 or p1 <= p0, else as af_patch_step_tiled and af_pack_owned. */
+typedef struct {
+    int32_t p0, p1;
+    int32_t nwork;
+    int32_t pad_;
+    const af_work *d_work;
+} af_band;
+af_status af_step_host_bands(const af_config *cfg, int32_t tiling, int32_t nband, const af_band *h_band, int32_t owned,
+                             void *h_state, void *d_up, void *d_down, void *d_a, void *d_b, double dt0, double dx0,
+                             double dy0, double *d_flux_reg, void *stream, void *s_in, void *s_cmp, void *s_out);
+
 /* Measurement probe (no counterpart in the paper): `blocks` CTAs of
  * af_fma_probe_threads() / 8 threads each run 8 independent fused
  * multiply-add chains of `iters` steps in precision `prec` (af_precision) and

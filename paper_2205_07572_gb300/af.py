@@ -111,10 +111,21 @@ def ptr(x):
     return x.data_ptr()
 
 
+_torch_c = None  # torch._C, once CUDA is initialised
+
+
 def stream_handle(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        # the current stream's handle straight from torch's bindings:
+        # torch.cuda.current_stream() builds an object after several look-ups,
+        # 3 us of a call that otherwise takes 6
+        global _torch_c
+        if _torch_c is None:
+            import torch
+            handle = torch.cuda.current_stream().cuda_stream
+            _torch_c = torch._C
+            return handle
+        return _torch_c._cuda_getCurrentRawStream(_torch_c._cuda_getDevice())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -469,6 +480,26 @@ _EXTRA += [("af_pack_owned", C.c_int, [C.POINTER(Config), C.c_int32, _VP, _VP, _
            ("af_unpack_owned", C.c_int, [C.POINTER(Config), C.c_int32, _VP, _VP, _VP])]
 if _lib is not None:
     _register_more(_lib)
+
+
+class Band(C.Structure):
+    """af_band: patches [p0, p1) and their device work list."""
+    _fields_ = [("p0", C.c_int32), ("p1", C.c_int32), ("nwork", C.c_int32), ("pad_", C.c_int32), ("d_work", C.c_void_p)]
+
+
+_EXTRA += [("af_step_host_bands", C.c_int, [C.POINTER(Config), C.c_int32, C.c_int32, C.POINTER(Band), C.c_int32, _VP, _VP,
+                                            _VP, _VP, _VP, C.c_double, C.c_double, C.c_double, _VP, _VP, _VP, _VP, _VP])]
+if _lib is not None:
+    _register_more(_lib)
+
+
+def step_host_bands(cfg: Config, tiling: int, bands, owned: bool, host, up, down, a, b, dt: float, dx: float, dy: float,
+                    flux_reg, stream, s_in, s_cmp, s_out) -> None:
+    """af_step_host_bands; bands: a ctypes array of Band."""
+    _check(lib().af_step_host_bands(C.byref(cfg), int(tiling), len(bands), bands, 1 if owned else 0, ptr(host), ptr(up),
+                                    ptr(down), ptr(a), ptr(b), float(dt), float(dx), float(dy), ptr(flux_reg),
+                                    stream_handle(stream), stream_handle(s_in), stream_handle(s_cmp),
+                                    stream_handle(s_out)), "af_step_host_bands")
 
 
 def owned_words(n: int, ncomp: int) -> int:

@@ -134,8 +134,29 @@ class UniformRun:
                 p = np.arange(edges[b] * self.px, edges[b + 1] * self.px)
                 w = af.build_step_work(self.cfg, p, nbr=self.nbr[p], tiling=self.tiling)
                 self._bands.append((int(p[0]), int(p[-1]) + 1, torch.from_numpy(w).to(self.device), len(w) // 64))
+            self._bands_c = (af.Band * bands)(*[af.Band(p0, p1, nw, 0, w.data_ptr()) for p0, p1, w, nw in self._bands])
             self._streams = [torch.cuda.Stream() for _ in range(3)]
+            self._mark = torch.empty(1, dtype=self.a.dtype, device=self.device)
             self._bands_key = key
+
+    def _step_host_native(self, host, words: int, up, down) -> bool:
+        """The banded step enqueued by one native call, if `host` is what that
+        takes: a CPU tensor of the state's type and exactly its shape, dense.
+        Anything else (another type, strides, broadcasting) goes through
+        torch's copies."""
+        import torch
+        if not (isinstance(host, torch.Tensor) and host.device.type == "cpu" and host.dtype == self.a.dtype
+                and host.shape == (self.npatch, words) and host.is_contiguous()):
+            return False
+        s_in, s_cmp, s_out = self._streams
+        af.step_host_bands(self.cfg, self.tiling, self._bands_c, up is not None, host, up, down, self.a, self.b, self.dt,
+                           self.dx, self.dy, self.freg, None, s_in, s_cmp, s_out)
+        # one element through torch on the caller's stream, which now waits for
+        # every copy of `host`: torch's allocator then knows until when the pinned
+        # block is in use
+        self._mark.copy_(host.view(-1)[:1], non_blocking=True)
+        self.t += self.dt
+        return True
 
     def step_host(self, host, bands: int = 16):
         """One step of a state kept in (pinned) host memory, updated in place:
@@ -150,6 +171,8 @@ class UniformRun:
             raise ValueError("step_host runs constant-velocity steps")
         bands = max(1, min(int(bands), self.py))
         self._band_setup(bands)
+        if self._step_host_native(host, self.words, None, None):
+            return
         s_in, s_cmp, s_out = self._streams
         cur = torch.cuda.current_stream()
         for st in self._streams:
@@ -197,6 +220,8 @@ class UniformRun:
             self._own_bufs = (torch.empty((self.npatch, words), dtype=self.a.dtype, device=self.device),
                               torch.empty((self.npatch, words), dtype=self.a.dtype, device=self.device))
         own_in, own_out = self._own_bufs
+        if self._step_host_native(host, words, own_in, own_out):
+            return
         s_in, s_cmp, s_out = self._streams
         cur = torch.cuda.current_stream()
         for st in self._streams:

@@ -1,5 +1,6 @@
 """CPU checks of the C ABI: the library loads, exports every declared entry
 point, and rejects bad arguments on the host before touching the GPU."""
+import ctypes as C
 import os
 import re
 
@@ -201,3 +202,17 @@ def test_mass_noalloc_host_side_errors_and_capacity(af):
     for nleaf in (1, 255, 256, 300, 1 << 20, (1 << 31) - 1):
         assert af.mass_scratch_bytes(nleaf, 3) <= 1024 * 8
     assert af.mass_scratch_bytes(1 << 20, 3) == 256 * 3 * 8
+
+
+def test_host_bands_refuse_bad_arguments(af):
+    """af_step_host_bands checks its arguments before anything is enqueued."""
+    cfg = af.config(af.ACOUSTICS, af.F32, 16)
+    ok = (af.Band * 1)(af.Band(0, 4, 0, 0, None))
+    call = lambda c=cfg, bands=ok, nband=1, host=64, up=64, down=64, a=64, b=128: af.lib().af_step_host_bands(  # noqa: E731
+        C.byref(c), 4, nband, bands, 1, host, up, down, a, b, 0.1, 1.0, 1.0, None, None, None, None, None)
+    assert call(nband=0) == 1 and call(host=None) == 1 and call(up=None) == 1 and call(a=None) == 1 and call(b=None) == 1
+    assert call(bands=None) == 1
+    assert call(bands=(af.Band * 1)(af.Band(3, 3, 0, 0, None))) == 1
+    assert call(bands=(af.Band * 1)(af.Band(-1, 3, 0, 0, None))) == 1
+    bad = af.config(af.ACOUSTICS, af.F32, 65)
+    assert call(c=bad) == 1

@@ -604,6 +604,48 @@ def test_host_owned_step_matches_device_step(af, bands):
     assert np.array_equal(host.numpy(), own.cpu().numpy())
 
 
+@pytest.mark.parametrize("owned", [False, True])
+@pytest.mark.parametrize("prec,bands,form", [(1, 3, "plain"), (0, 8, "plain"), (1, 4, "strided"), (1, 3, "double"),
+                                             (0, 2, "pageable"), (1, 2, "other_stream")])
+def test_host_step_takes_every_form_of_host_state(af, owned, prec, bands, form):
+    """The banded host steps give the device step's owned entries bit for bit
+    whatever the host tensor: dense and of the state's type (one native call),
+    pageable, strided, of another type (torch's copies), and from a stream of
+    the caller's own."""
+    from paper_2205_07572_gb300.uniform import UniformRun
+    n, px, nc = 8, 8, 3
+    grid = S.UniformGrid(S.Layout(n, nc), px, px)
+    st = S.periodic_state(grid, S.pulse_plus_vortex(), nq=2)
+    cfg = af.config(af.ACOUSTICS, prec, n, c=1.0)
+    dev = UniformRun(cfg, px, px, grid.dx, grid.dy, 0.4 * grid.dx, state=st)
+    hrun = UniformRun(cfg, px, px, grid.dx, grid.dy, 0.4 * grid.dx, state=None)
+    own = torch.empty((grid.npatch, af.owned_words(n, nc)), dtype=dev.a.dtype, device="cuda")
+
+    def owned_of(state):
+        af.pack_owned(cfg, grid.npatch, state, own)
+        torch.cuda.synchronize()
+        return own.cpu().numpy().copy()
+
+    src = torch.from_numpy(owned_of(dev.a)) if owned else dev.a.cpu()
+    if form == "strided":
+        host = torch.empty((src.shape[0], 2 * src.shape[1]), dtype=src.dtype, pin_memory=True)[:, ::2]
+        host.copy_(src)
+    elif form == "double":
+        host = src.double().pin_memory()
+    else:
+        host = src.clone() if form == "pageable" else src.clone().pin_memory()
+    side = torch.cuda.Stream()
+    for _ in range(3):
+        dev.step()
+        with torch.cuda.stream(side if form == "other_stream" else torch.cuda.current_stream()):
+            (hrun.step_host_owned if owned else hrun.step_host)(host, bands)
+    torch.cuda.synchronize()
+    ref = owned_of(dev.a)
+    got = host.to(dev.a.dtype).contiguous().numpy() if owned else owned_of(host.to(dev.a.dtype).cuda())
+    assert np.array_equal(got, ref)
+    assert hrun.t == dev.t
+
+
 @pytest.mark.parametrize("prec", [0, 1])
 def test_fma_probe_computes_its_chains(af, prec):
     """af_fma_throughput (the ALU-roof probe) runs the chains it claims: every
