@@ -14,6 +14,7 @@
 #include <cstring>
 
 #include "af_internal.h"
+#include "af_launch.cuh"
 
 namespace af {
 namespace {
@@ -602,7 +603,8 @@ __global__ void __launch_bounds__(256) plan_build_kernel(const __grid_constant__
 template <typename T>
 __global__ void plan_exec_a(StateView<T> S, const GhostEntry *__restrict__ plan, long long na, uint32_t levels,
                             int same_only) {
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < na; t += (long long)gridDim.x * blockDim.x) {
+    const unsigned block = chain_begin();
+    for (long long t = block * (long long)blockDim.x + threadIdx.x; t < na; t += (long long)gridDim.x * blockDim.x) {
         const GhostEntry g = plan[t];
         const int ld = g.levels & 15, ls = g.levels >> 4;
         if (!((levels >> ld) & 1u) || !((levels >> ls) & 1u) || (same_only && ld != ls)) continue;
@@ -623,7 +625,8 @@ __global__ void plan_exec_a(StateView<T> S, const GhostEntry *__restrict__ plan,
 
 template <typename T>
 __global__ void plan_exec_b(StateView<T> S, int n, const GhostEntry *__restrict__ plan, long long nb, uint32_t levels) {
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nb; t += (long long)gridDim.x * blockDim.x) {
+    const unsigned block = chain_begin();
+    for (long long t = block * (long long)blockDim.x + threadIdx.x; t < nb; t += (long long)gridDim.x * blockDim.x) {
         const GhostEntry g = plan[t];
         const int ld = g.levels & 15, ls = g.levels >> 4;
         if (!((levels >> ld) & 1u) || !((levels >> ls) & 1u)) continue;
@@ -808,7 +811,8 @@ template <typename T>
 __global__ void reflux_kernel(const __grid_constant__ DevForest F, StateView<T> S, uint32_t sync, double dx0, double dy0, double *freg) {
     const int n = F.n, nc = S.ncomp;
     const int64_t total = (int64_t)F.nleaf * 4 * n;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned block = chain_begin();
+    for (int64_t t = block * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
         // 32-bit divisions (total < 2^31 for any state that fits the GPU)
         const int f = (int)t / n, k = (int)t - f * n, p = f >> 2, side = f & 3;
         const int l = __ldg(F.level + p);
@@ -1093,21 +1097,18 @@ extern "C" af_status af_fill_ghosts_planned(const af_config *cfg, const af_fores
     const GhostEntry *plan = static_cast<const GhostEntry *>(d_plan);
     const int same = (flags & AF_FILL_SAME_LEVEL_ONLY) ? 1 : 0;
     auto grid = [](int64_t m) { return (int)(m / 256 + 1 < 152 * 16 ? m / 256 + 1 : 152 * 16); };
+    const bool chain = cfg->prec == AF_F32 || cfg->eq == AF_ADVECTION;  // as the step between two exchanges
     if (n_a > 0) {
-        if (cfg->prec == AF_F64)
-            plan_exec_a<double><<<grid(n_a), 256, 0, s>>>(view<double>(*cfg, *forest, *state), plan, n_a, levels, same);
-        else
-            plan_exec_a<float><<<grid(n_a), 256, 0, s>>>(view<float>(*cfg, *forest, *state), plan, n_a, levels, same);
-        if (launched() != AF_OK) return AF_ERR_CUDA;
+        const cudaError_t e = cfg->prec == AF_F64
+            ? launch_chained(chain, plan_exec_a<double>, grid(n_a), 256, 0, s, view<double>(*cfg, *forest, *state), plan, n_a, levels, same)
+            : launch_chained(chain, plan_exec_a<float>, grid(n_a), 256, 0, s, view<float>(*cfg, *forest, *state), plan, n_a, levels, same);
+        if (e != cudaSuccess) return AF_ERR_CUDA;
     }
     if (n_b > 0 && !same) {
-        if (cfg->prec == AF_F64)
-            plan_exec_b<double><<<grid(n_b), 256, 0, s>>>(view<double>(*cfg, *forest, *state), cfg->n, plan + n_a, n_b,
-                                                         levels);
-        else
-            plan_exec_b<float><<<grid(n_b), 256, 0, s>>>(view<float>(*cfg, *forest, *state), cfg->n, plan + n_a, n_b,
-                                                        levels);
-        if (launched() != AF_OK) return AF_ERR_CUDA;
+        const cudaError_t e = cfg->prec == AF_F64
+            ? launch_chained(chain, plan_exec_b<double>, grid(n_b), 256, 0, s, view<double>(*cfg, *forest, *state), cfg->n, plan + n_a, n_b, levels)
+            : launch_chained(chain, plan_exec_b<float>, grid(n_b), 256, 0, s, view<float>(*cfg, *forest, *state), cfg->n, plan + n_a, n_b, levels);
+        if (e != cudaSuccess) return AF_ERR_CUDA;
     }
     return AF_OK;
 }
@@ -1152,13 +1153,11 @@ extern "C" af_status af_reflux_pair(const af_config *cfg, const af_forest *fores
     const DevForest F = make_dev(*forest, cfg->n);
     const long long total = (long long)forest->nleaf * 4 * cfg->n;
     const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-    if (cfg->prec == AF_F64)
-        reflux_kernel<double><<<blocks, 256, 0, s>>>(F, view<double>(*cfg, *forest, *state), sync_levels, dx0, dy0,
-                                                     d_flux_reg);
-    else
-        reflux_kernel<float><<<blocks, 256, 0, s>>>(F, view<float>(*cfg, *forest, *state), sync_levels, dx0, dy0,
-                                                    d_flux_reg);
-    return launched();
+    const bool chain = cfg->prec == AF_F32 || cfg->eq == AF_ADVECTION;  // as the step before the fix
+    const cudaError_t e = cfg->prec == AF_F64
+        ? launch_chained(chain, reflux_kernel<double>, blocks, 256, 0, s, F, view<double>(*cfg, *forest, *state), sync_levels, dx0, dy0, d_flux_reg)
+        : launch_chained(chain, reflux_kernel<float>, blocks, 256, 0, s, F, view<float>(*cfg, *forest, *state), sync_levels, dx0, dy0, d_flux_reg);
+    return e == cudaSuccess ? AF_OK : AF_ERR_CUDA;
 }
 
 extern "C" af_status af_reflux(const af_config *cfg, const af_forest *forest, uint32_t sync_levels, double dx0,

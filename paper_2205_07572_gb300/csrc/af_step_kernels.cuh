@@ -29,6 +29,7 @@
 #include <cuda_runtime.h>
 
 #include "af_internal.h"
+#include "af_launch.cuh"
 
 namespace af {
 
@@ -196,6 +197,10 @@ __device__ __forceinline__ void quad(T pp, T pm, T mp, T mm, T &ss, T &as, T &sa
     as = a - b;
     sa = (pp - pm) + (mp - mm);
 }
+
+// A product rounded on its own (never contracted into a sum).
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
 // acc += w . v as one chain of fused multiply-adds
 template <int N, typename T>
@@ -533,8 +538,9 @@ __device__ __forceinline__ void tile_nodes(const StepArgs<T> &A, const typename 
 
 // Fluxes (Eq. Simpson-2d) and the update (Eq. 2dfv) of one tile whose T
 // arrays tile_nodes has written; reads the cell averages from the window.
-// FREG: A.freg is set (adaptive runs); the flux registers of patch-boundary
-// cells are accumulated.
+// FREG: adaptive runs, whose flux registers take the rounded face fluxes: in
+// FP32 the update takes the same ones, rounded before their difference (uniform
+// runs and FP64 leave one product in the difference's multiply-add).
 template <typename T, int EQ, int NT, int WX, int WSZ, int TX, int TSZ, int TMX, int NN, bool FREG>
 __device__ __forceinline__ void tile_fluxes(const StepArgs<T> &A, const T *Sin, const T *ST, int patch, int level,
                                             int x0, int x1, int y0, int y1) {
@@ -557,23 +563,6 @@ __device__ __forceinline__ void tile_fluxes(const StepArgs<T> &A, const T *Sin, 
         }
         const int i = x0 + ii, j = y0 + jj;
         const int s00 = jj * TX + ii;
-        // flux registers of a patch-boundary cell: its x side (0 left, 1
-        // right) and y side (2 bottom, 3 top), read first so their latency
-        // overlaps the flux arithmetic (each entry belongs to one cell)
-        double *fr_p = nullptr;
-        int kx = -1, ky = -1;
-        double ox[3], oy[3];
-        if (FREG) {
-            fr_p = A.freg + (int64_t)patch * 4 * ncomp * n;
-            const bool iny = (j >= 0 && j < n), inx = (i >= 0 && i < n);
-            kx = (iny && i == 0) ? 0 : ((iny && i == n - 1) ? 1 : -1);
-            ky = (inx && j == 0) ? 2 : ((inx && j == n - 1) ? 3 : -1);
-#pragma unroll
-            for (int c = 0; c < ncomp; ++c) {
-                if (kx >= 0) ox[c] = fr_p[(kx * ncomp + c) * n + j];
-                if (ky >= 0) oy[c] = fr_p[(ky * ncomp + c) * n + i];
-            }
-        }
         T Fl[3], Fr[3], Gb[3], Gt[3];
 #pragma unroll
         for (int c = 0; c < ncomp; ++c) {
@@ -586,15 +575,16 @@ __device__ __forceinline__ void tile_fluxes(const StepArgs<T> &A, const T *Sin, 
             Gt[c] = fma(T(4), Ty[s00 + TX], Tc[s00 + TX]) + Tc[s00 + TX + 1];
         }
         T fl[3], fr[3], gb[3], gt[3];
+        auto flux = [](T k, T s) { return FREG && sizeof(T) == 4 ? mul_rn(k, s) : k * s; };
         if constexpr (EQ == AF_ACOUSTICS) {
             // f = c (u, p, 0), g = c (v, 0, p)
-            fl[0] = A.fx * Fl[1]; fl[1] = A.fx * Fl[0]; fl[2] = T(0);
-            fr[0] = A.fx * Fr[1]; fr[1] = A.fx * Fr[0]; fr[2] = T(0);
-            gb[0] = A.fy * Gb[2]; gb[1] = T(0); gb[2] = A.fy * Gb[0];
-            gt[0] = A.fy * Gt[2]; gt[1] = T(0); gt[2] = A.fy * Gt[0];
+            fl[0] = flux(A.fx, Fl[1]); fl[1] = flux(A.fx, Fl[0]); fl[2] = T(0);
+            fr[0] = flux(A.fx, Fr[1]); fr[1] = flux(A.fx, Fr[0]); fr[2] = T(0);
+            gb[0] = flux(A.fy, Gb[2]); gb[1] = T(0); gb[2] = flux(A.fy, Gb[0]);
+            gt[0] = flux(A.fy, Gt[2]); gt[1] = T(0); gt[2] = flux(A.fy, Gt[0]);
         } else {
-            fl[0] = A.fx * Fl[0]; fr[0] = A.fx * Fr[0];
-            gb[0] = A.fy * Gb[0]; gt[0] = A.fy * Gt[0];
+            fl[0] = flux(A.fx, Fl[0]); fr[0] = flux(A.fx, Fr[0]);
+            gb[0] = flux(A.fy, Gb[0]); gt[0] = flux(A.fy, Gt[0]);
         }
         T *const ob = outp + ((j + kGhost) * W_ + (i + kGhost));
         const int sa = (jj + 1) * WX + (ii + 1);
@@ -605,18 +595,67 @@ __device__ __forceinline__ void tile_fluxes(const StepArgs<T> &A, const T *Sin, 
             const T q = Sin[(c * kPlanes + kAvg) * WSZ + sa];
             __stcs(ob + c * kPlanes * plane, fma(-A.dtdy, gt[c] - gb[c], fma(-A.dtdx, fr[c] - fl[c], q)));
         }
-        if (FREG) {
-            // dt_l = dt0 / 2^level, scaled exactly by the power of two (no FP64
-            // library call outside this branch)
-            const double dtl = A.dt0 * __longlong_as_double((long long)(1023 - level) << 52);
-#pragma unroll
-            for (int c = 0; c < ncomp; ++c) {
-                if (kx >= 0) fr_p[(kx * ncomp + c) * n + j] = ox[c] + dtl * (double)(kx == 0 ? fl[c] : fr[c]);
-                if (ky >= 0) fr_p[(ky * ncomp + c) * n + i] = oy[c] + dtl * (double)(ky == 2 ? gb[c] : gt[c]);
-            }
-        }
     }
 }
+
+// Adaptive runs: dt_l F of the tile's faces on the patch boundary, added to the
+// FP64 flux registers.  One value per thread and turn -- the components whose
+// flux is not identically zero, along each side -- read before the flux loop
+// and stored after it, so that the registers' latency hides behind the loop.
+// (In the loop itself, two lanes of every warp took all warps through the FP64
+// multiply-adds of both x sides: 60 warp instructions of that pipe for a
+// 16 x 16 tile, 8 now.  Adaptive acoustics on 5436 leaves 1317 -> 1237 us a
+// coarse step.)
+template <typename T, int EQ, int NT, int TX, int TSZ, int NN>
+struct BoundaryFluxes {
+    static constexpr int ncomp = (EQ == AF_ACOUSTICS) ? 3 : 1, nz = (EQ == AF_ACOUSTICS) ? 2 : 1;
+    static constexpr int kHeld = 2;  // values a thread holds over the flux loop (a 32 x 32 patch on 128 threads)
+    double *reg[kHeld];
+    double old[kHeld];
+    T flux[kHeld];
+
+    // Value t of the tile: its register, and its flux from the T arrays; null
+    // if the face is not in the tile.
+    static __device__ __forceinline__ double *value(const StepArgs<T> &A, const T *ST, int patch, int x0, int x1, int y0,
+                                                    int y1, int t, T &f) {
+        const int n = NN > 0 ? NN : A.n;
+        const int q = nz * n, side = (t >= q) + (t >= 2 * q) + (t >= 3 * q), r = t - side * q;
+        const int z = nz == 2 && r >= n ? 1 : 0, k = r - z * n;
+        const bool xs = side < 2;
+        const int line = (side & 1) ? n : 0, cell = (side & 1) ? n - 1 : 0;  // the face's node line, its cell inside
+        const int lo = xs ? x0 : y0, hi = xs ? x1 : y1, klo = xs ? y0 : x0, khi = xs ? y1 : x1;
+        if (cell < lo || cell >= hi || k < klo || k >= khi) return nullptr;
+        // f = c (u, p, 0), g = c (v, 0, p): component c of the flux is value v
+        const int c = EQ == AF_ACOUSTICS ? (xs ? z : 2 * z) : 0;
+        const int v = EQ == AF_ACOUSTICS ? (xs ? 1 - z : 2 - 2 * z) : 0;
+        const int s = xs ? (k - y0) * TX + (line - x0) : (line - y0) * TX + (k - x0);
+        const T *const Tc = ST + v * 3 * TSZ + s, *const Tm = Tc + (xs ? 1 : 2) * TSZ;
+        f = mul_rn(xs ? A.fx : A.fy, fma(T(4), Tm[0], Tc[0]) + Tc[xs ? TX : 1]);
+        return A.freg + ((int64_t)patch * 4 + side) * ncomp * n + c * n + k;
+    }
+    __device__ __forceinline__ void begin(const StepArgs<T> &A, const T *ST, int patch, int x0, int x1, int y0, int y1) {
+#pragma unroll
+        for (int h = 0; h < kHeld; ++h) {
+            const int t = threadIdx.x + h * NT, total = 4 * nz * (NN > 0 ? NN : A.n);
+            reg[h] = t < total ? value(A, ST, patch, x0, x1, y0, y1, t, flux[h]) : nullptr;
+            if (reg[h]) old[h] = *reg[h];
+        }
+    }
+    __device__ __forceinline__ void end(const StepArgs<T> &A, const T *ST, int patch, int level, int x0, int x1, int y0,
+                                        int y1) {
+        // dt_l = dt0 / 2^level, scaled exactly by the power of two
+        const double dtl = A.dt0 * __longlong_as_double((long long)(1023 - level) << 52);
+        const int total = 4 * nz * (NN > 0 ? NN : A.n);
+#pragma unroll
+        for (int h = 0; h < kHeld; ++h)
+            if (reg[h]) *reg[h] = old[h] + dtl * (double)flux[h];
+        for (int t = threadIdx.x + kHeld * NT; t < total; t += NT) {
+            T f;
+            double *const p = value(A, ST, patch, x0, x1, y0, y1, t, f);
+            if (p) *p += dtl * (double)f;
+        }
+    }
+};
 
 // Point values, then fluxes and update, of one staged tile.
 template <typename T, int EQ, int NT, int WX, int WSZ, int TX, int TSZ, int TMX = TX - 1, int NN = 0>
@@ -627,10 +666,14 @@ __device__ __forceinline__ void tile_compute(const StepArgs<T> &A, const typenam
     __syncthreads();
     // flux registers (adaptive runs) or none: two instantiations, so the
     // uniform grid's loop carries nothing of them
-    if (A.freg != nullptr)
+    if (A.freg != nullptr) {
+        BoundaryFluxes<T, EQ, NT, TX, TSZ, NN> B;
+        B.begin(A, ST, patch, x0, x1, y0, y1);
         tile_fluxes<T, EQ, NT, WX, WSZ, TX, TSZ, TMX, NN, true>(A, Sin, ST, patch, level, x0, x1, y0, y1);
-    else
+        B.end(A, ST, patch, level, x0, x1, y0, y1);
+    } else {
         tile_fluxes<T, EQ, NT, WX, WSZ, TX, TSZ, TMX, NN, false>(A, Sin, ST, patch, level, x0, x1, y0, y1);
+    }
 }
 
 // Resident CTAs per SM the register allocation must allow: FP32 acoustics
@@ -1000,8 +1043,9 @@ __global__ void __launch_bounds__(NT, (min_ctas<T, EQ, NT>())) step_kernel(const
     T *const Sbase = reinterpret_cast<T *>(smem_raw);
     T *Sin = Sbase + win_off<T, Gm::WX>();
     T *ST = Sbase + ncomp * kPlanes * Gm::WSZ;
-    prefetch_work(A.work, blockIdx.x + kWorkPrefetch, gridDim.x);
-    af_work wk = load_work(A.work + blockIdx.x);
+    const unsigned block = chain_begin();
+    prefetch_work(A.work, block + kWorkPrefetch, gridDim.x);
+    af_work wk = load_work(A.work + block);
     if (wk.x1 - wk.x0 > TMX || wk.y1 - wk.y0 > TMY) return;  // built for another tiling
     if constexpr (SPLIT) {
         // (a tile whose copies are made to fail stays whole: one wait runs out)
@@ -1132,12 +1176,13 @@ __global__ void __launch_bounds__(NT, (min_ctas<T, EQ, NT>())) step_kernel_pipe(
             cp_async_commit();
         }
         if (fits) {
-            if (A.freg != nullptr)
-                tile_fluxes<T, EQ, NT, Gm::WX, Gm::WSZ, Gm::TX, Gm::TSZ, TMX, NN, true>(A, Sc, ST, wk.patch, wk.level,
-                                                                                       wk.x0, wk.x1, wk.y0, wk.y1);
-            else
-                tile_fluxes<T, EQ, NT, Gm::WX, Gm::WSZ, Gm::TX, Gm::TSZ, TMX, NN, false>(A, Sc, ST, wk.patch, wk.level,
-                                                                                        wk.x0, wk.x1, wk.y0, wk.y1);
+            tile_fluxes<T, EQ, NT, Gm::WX, Gm::WSZ, Gm::TX, Gm::TSZ, TMX, NN, true>(A, Sc, ST, wk.patch, wk.level, wk.x0, wk.x1,
+                                                                              wk.y0, wk.y1);
+            if (A.freg != nullptr) {
+                BoundaryFluxes<T, EQ, NT, Gm::TX, Gm::TSZ, NN> B;
+                B.begin(A, ST, wk.patch, wk.x0, wk.x1, wk.y0, wk.y1);
+                B.end(A, ST, wk.patch, wk.level, wk.x0, wk.x1, wk.y0, wk.y1);
+            }
             if (bulk_tile<T, Gm::WX>(A, wk)) write_ghost_columns<T, NT, Gm::WX, Gm::WSZ, ncomp>(A, wk, Sc);
         }
         cp_async_wait_all();
@@ -1188,6 +1233,7 @@ af_status launch_tiling(const StepArgs<T> &A, const typename WeightsOf<T, EQ>::t
         (void)tarr;
         return AF_ERR_UNIMPLEMENTED;
     } else {
+        constexpr bool chain = sizeof(T) == 4 || EQ == AF_ADVECTION;
         const size_t smem = win + tarr;
         if (smem > 227 * 1024) return AF_ERR_UNIMPLEMENTED;
         if constexpr (NN == 0) {
@@ -1195,15 +1241,14 @@ af_status launch_tiling(const StepArgs<T> &A, const typename WeightsOf<T, EQ>::t
             if (split > 1) {
                 auto kern = dev::step_kernel<T, EQ, NT, TMX, TMY, 0, true>;
                 if (ensure_smem(kern, smem) != cudaSuccess) return AF_ERR_CUDA;
-                kern<<<dim3(nwork, split), NT, smem, stream>>>(A, W);
-                return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+                return launch_chained(chain, kern, dim3(nwork, split), NT, smem, stream, A, W) == cudaSuccess ? AF_OK
+                                                                                                     : AF_ERR_CUDA;
             }
         }
         auto kern = dev::step_kernel<T, EQ, NT, TMX, TMY, NN>;
         if (ensure_smem(kern, smem) != cudaSuccess) return AF_ERR_CUDA;
-        kern<<<nwork, NT, smem, stream>>>(A, W);
+        return launch_chained(chain, kern, nwork, NT, smem, stream, A, W) == cudaSuccess ? AF_OK : AF_ERR_CUDA;
     }
-    return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
 }
 
 #define AF_TILING_CASE(K)                                                                                 \

@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 768 / NT : 1) step_var_ke
     // the sine and cosine of 2 pi x (swirl), or x itself in .s (solid body)
     __shared__ SC<T> tx[2][TMX + 1], ty[2][TMY + 1];
     const StepArgs<T> &A = V.s;
-    const af_work wk = load_work(A.work + blockIdx.x);
+    const af_work wk = load_work(A.work + chain_begin());
     if (wk.x1 - wk.x0 > TMX || wk.y1 - wk.y0 > TMY) return;
     const int n = NN > 0 ? NN : A.n, W_ = n + 2 * kGhost + 1, level = wk.level;
     const int plane = NN > 0 ? (int)plane_stride(NN) : (int)A.plane;
@@ -339,8 +339,7 @@ af_status launch_var_kernel(const VarArgs<T> &V, int nwork, cudaStream_t stream)
     if (smem > 227 * 1024) return AF_ERR_UNIMPLEMENTED;
     auto kern = step_var_kernel<T, FIELD, MODE, NT, TMX, TMY, NN>;
     if (ensure_smem(kern, smem) != cudaSuccess) return AF_ERR_CUDA;
-    kern<<<nwork, NT, smem, stream>>>(V);
-    return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+    return launch_chained(true, kern, nwork, NT, smem, stream, V) == cudaSuccess ? AF_OK : AF_ERR_CUDA;
 }
 
 // A tiling two cells wider than a patch (8 x 8 and 16 x 16 patches with their
