@@ -345,6 +345,36 @@ def _resplit(work, n, cuts):
     return np.ascontiguousarray(np.stack(out)).view(np.uint8).reshape(-1)
 
 
+@pytest.mark.parametrize("eq,prec", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("n,px", [(16, 2), (32, 16)])
+def test_chained_steps_see_what_ran_before_them(af, eq, prec, n, px):
+    """Steps are launched while the kernel before them is still finishing and
+    wait for it on the device: a long run of steps with kernels of torch between
+    them that change the state, on a stream of their own, equals the same run
+    with a synchronisation after every operation, bit for bit."""
+    from paper_2205_07572_gb300.uniform import UniformRun
+    nc = 1 if eq == 0 else 3
+    grid = S.UniformGrid(S.Layout(n, nc), px, px)
+    st = np.nan_to_num(S.pack_owned(grid, S.random_owned(grid, seed=n)))
+    ends = []
+    for sync in (False, True):
+        run = UniformRun(af.config(eq, prec, n, 0.9, -0.4, 1.0), px, px, grid.dx, grid.dy, 0.4 * grid.dx, state=st)
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            for k in range(40):
+                run.step()
+                if sync:
+                    torch.cuda.synchronize()
+                if k % 3 == 0:
+                    run.state.mul_(0.75)
+                    if sync:
+                        torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        ends.append(S.unpack_owned(grid, run.state.double().cpu().numpy().reshape(st.shape)))
+    assert np.isfinite(ends[0]).all() and np.array_equal(ends[0], ends[1])
+
+
 @pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("a,b", [(0.45, 0.3), (-0.5, 0.5), (0.0, -0.45), (0.95, 0.2), (-0.3, -1.0), (0.6, 0.7), (1.0, 0.0)])
 @pytest.mark.parametrize("n,px,py", [(16, 2, 3), (23, 2, 1), (32, 1, 2)])
