@@ -1252,8 +1252,8 @@ inline cudaError_t ensure_smem(Kern k, size_t bytes) {
 // SPLIT): one, unless the tiles leave most of the GPU's 152 SMs idle.  Then as
 // many as bring two CTAs to an SM, of two rows or more: a band's extra row of
 // nodes costs up to half its work again, on SMs that would do nothing.  One
-// 64 x 64 FP64 patch in 32 x 32 tiles: 28.7 us on four CTAs, 9.2 us (the host's
-// share of a call) on 64.
+// 64 x 64 FP64 patch in 32 x 32 tiles: 28.7 us on four CTAs, 9.2 us on 64,
+// where the host's share of a call set the time (5.2 us since that shrank).
 inline int few_tiles(int nwork, int rows) {
     const int s = 2 * 152 / (nwork < 1 ? 1 : nwork), most = rows / 2;
     return s < 2 ? 1 : (s < most ? s : (most < 1 ? 1 : most));
