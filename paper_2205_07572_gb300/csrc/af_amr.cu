@@ -669,8 +669,61 @@ __global__ void __launch_bounds__(256, 6) plan_exec_a3(StateView<T> S, const Gho
     }
 }
 
-template <typename T>
-__global__ void plan_exec_b(StateView<T> S, int n, const GhostEntry *__restrict__ plan, long long nb, uint32_t levels) {
+// Pass B in FP32.  Few entries, each a chain: the entry, then nine values of the
+// coarser leaf per component.  All NC components' values are read before one is
+// written, and nothing is computed in FP64 (positions in a cell are multiples of
+// a half: exact in either).  Adaptive acoustics on 5436 leaves 1157 -> 1135 us a
+// coarse step, advection on 2944 leaves 184 -> 179.
+template <int NC>
+__global__ void __launch_bounds__(256) plan_exec_b(StateView<float> S, int n, const GhostEntry *__restrict__ plan, long long nb,
+                                                   uint32_t levels) {
+    using T = float;
+    const unsigned block = chain_begin();
+    for (long long t = block * (long long)blockDim.x + threadIdx.x; t < nb; t += (long long)gridDim.x * blockDim.x) {
+        const GhostEntry g = plan[t];
+        const int ld = g.levels & 15, ls = g.levels >> 4;
+        if (!((levels >> ld) & 1u) || !((levels >> ls) & 1u)) continue;
+        T *dst = S.patch_at_level(g.dst, ld) + g.dst_off;
+        const int u = (int)(g.aux & 0xffffu), v = (int)(g.aux >> 16);
+        const int64_t cs = (int64_t)kPlanes * S.plane;
+        const int W = S.W;
+        // the cell holding the quarter-cell position (u, v) of the source leaf,
+        // chosen as the direct exchange chooses it
+        int ci = u / 4, cj = v / 4;
+        ci = ci > n - 1 ? n - 1 : ci;
+        cj = cj > n - 1 ? n - 1 : cj;
+        const T *cell = S.patch_at_level(g.src, ls) + (int64_t)(cj + kGhost) * W + (ci + kGhost);
+        T w[NC][9], r[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const T *cr = cell + c * cs + kCorner * S.plane, *xm = cell + c * cs + kXmid * S.plane;
+            const T *ym = cell + c * cs + kYmid * S.plane, *av = cell + c * cs + kAvg * S.plane;
+            w[c][0] = cr[0], w[c][1] = cr[1], w[c][2] = cr[W], w[c][3] = cr[W + 1];
+            w[c][4] = xm[0], w[c][5] = xm[1], w[c][6] = ym[0], w[c][7] = ym[W], w[c][8] = av[0];
+        }
+        if (g.kind != kGPoint) {
+            // the mean over the quarter of the cell that (u, v), the centre of a
+            // cell one level finer, lies in
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                r[c] = recon_quarter_mean<T>(w[c][0], w[c][1], w[c][2], w[c][3], w[c][4], w[c][5], w[c][6], w[c][7], w[c][8],
+                                             u - 4 * ci >= 2, v - 4 * cj >= 2);
+        } else {
+            const T xi = (T)0.5 * (T)(u - 4 * ci) - (T)1, eta = (T)0.5 * (T)(v - 4 * cj) - (T)1;
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                r[c] = recon_eval<T>(w[c][0], w[c][1], w[c][2], w[c][3], w[c][4], w[c][5], w[c][6], w[c][7], w[c][8], xi, eta);
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) dst[c * cs] = r[c];
+    }
+}
+
+// Pass B in FP64, component by component: read ahead as above, acoustics were no
+// faster (levels 2-5, 671 us a coarse step either way) and advection slower (2944
+// leaves 1000 us, 1014).
+__global__ void plan_exec_b_f64(StateView<double> S, int n, const GhostEntry *__restrict__ plan, long long nb, uint32_t levels) {
+    using T = double;
     const unsigned block = chain_begin();
     for (long long t = block * (long long)blockDim.x + threadIdx.x; t < nb; t += (long long)gridDim.x * blockDim.x) {
         const GhostEntry g = plan[t];
@@ -853,9 +906,15 @@ __device__ __forceinline__ void atomic_add_state<double>(double *p, double v) { 
 template <>
 __device__ __forceinline__ void atomic_add_state<float>(float *p, double v) { atomicAdd(p, (float)v); }
 
-template <typename T>
+// A chain of loads per thread -- the leaf, its neighbour, the registers of both
+// -- on few threads, so its time is that chain's latency: the registers of all
+// NC components are read before any is written, which the compiler cannot
+// arrange itself (they may be the same as far as it knows).  Adaptive acoustics on
+// 5436 leaves 1161 -> 1157 us a coarse step, levels 3-7 with a ring per tree
+// 3996 -> 3980.
+template <typename T, int NC>
 __global__ void reflux_kernel(const __grid_constant__ DevForest F, StateView<T> S, uint32_t sync, double dx0, double dy0, double *freg) {
-    const int n = F.n, nc = S.ncomp;
+    const int n = F.n;
     const int64_t total = (int64_t)F.nleaf * 4 * n;
     const unsigned block = chain_begin();
     for (int64_t t = block * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
@@ -879,17 +938,24 @@ __global__ void reflux_kernel(const __grid_constant__ DevForest F, StateView<T> 
         if (kf < 0 || kf + 1 >= n) continue;
         const int ci = side == 0 ? 0 : (side == 1 ? n - 1 : k);
         const int cj = side == 2 ? 0 : (side == 3 ? n - 1 : k);
-        const double h = (side < 2 ? dx0 : dy0) / (double)(1LL << l);
-        const int64_t rw = 4LL * nc * n;
-        for (int c = 0; c < nc; ++c) {
-            double *rc = freg + p * rw + ((int64_t)side * nc + c) * n + k;
-            double *rf = freg + q * rw + ((int64_t)fside * nc + c) * n + kf;
-            const double fine = 0.5 * (rf[0] + rf[1]);
-            const double d = (side == 1 || side == 3) ? (*rc - fine) / h : (fine - *rc) / h;
+        const double h = (side < 2 ? dx0 : dy0) * __hiloint2double((1023 - l) << 20, 0);  // / 2^l, exactly
+        const int64_t rw = 4LL * NC * n;
+        double *rc = freg + p * rw + (int64_t)side * NC * n + k, *rf = freg + q * rw + (int64_t)fside * NC * n + kf;
+        double coarse[NC], f0[NC], f1[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            coarse[c] = rc[c * n];
+            f0[c] = rf[c * n];
+            f1[c] = rf[c * n + 1];
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const double fine = 0.5 * (f0[c] + f1[c]);
+            const double d = (side == 1 || side == 3) ? (coarse[c] - fine) / h : (fine - coarse[c]) / h;
             atomic_add_state<T>(S.at(p, c, kAvg, ci, cj), d);
-            *rc = 0.0;
-            rf[0] = 0.0;
-            rf[1] = 0.0;
+            rc[c * n] = 0.0;
+            rf[c * n] = 0.0;
+            rf[c * n + 1] = 0.0;
         }
     }
 }
@@ -1154,8 +1220,9 @@ extern "C" af_status af_fill_ghosts_planned(const af_config *cfg, const af_fores
     }
     if (n_b > 0 && !same) {
         const cudaError_t e = cfg->prec == AF_F64
-            ? launch_chained(chain, plan_exec_b<double>, grid(n_b), 256, 0, s, view<double>(*cfg, *forest, *state), cfg->n, plan + n_a, n_b, levels)
-            : launch_chained(chain, plan_exec_b<float>, grid(n_b), 256, 0, s, view<float>(*cfg, *forest, *state), cfg->n, plan + n_a, n_b, levels);
+            ? launch_chained(chain, plan_exec_b_f64, grid(n_b), 256, 0, s, view<double>(*cfg, *forest, *state), cfg->n, plan + n_a, n_b, levels)
+            : launch_chained(chain, cfg->ncomp == 3 ? plan_exec_b<3> : plan_exec_b<1>, grid(n_b), 256, 0, s,
+                             view<float>(*cfg, *forest, *state), cfg->n, plan + n_a, n_b, levels);
         if (e != cudaSuccess) return AF_ERR_CUDA;
     }
     return AF_OK;
@@ -1202,9 +1269,14 @@ extern "C" af_status af_reflux_pair(const af_config *cfg, const af_forest *fores
     const long long total = (long long)forest->nleaf * 4 * cfg->n;
     const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
     const bool chain = cfg->prec == AF_F32 || cfg->eq == AF_ADVECTION;  // as the step before the fix
-    const cudaError_t e = cfg->prec == AF_F64
-        ? launch_chained(chain, reflux_kernel<double>, blocks, 256, 0, s, F, view<double>(*cfg, *forest, *state), sync_levels, dx0, dy0, d_flux_reg)
-        : launch_chained(chain, reflux_kernel<float>, blocks, 256, 0, s, F, view<float>(*cfg, *forest, *state), sync_levels, dx0, dy0, d_flux_reg);
+    const auto run = [&](auto kernel, auto state_view) {
+        return launch_chained(chain, kernel, blocks, 256, 0, s, F, state_view, sync_levels, dx0, dy0, d_flux_reg);
+    };
+    const bool one = cfg->eq == AF_ADVECTION;
+    const cudaError_t e =
+        cfg->prec == AF_F64
+            ? run(one ? reflux_kernel<double, 1> : reflux_kernel<double, 3>, view<double>(*cfg, *forest, *state))
+            : run(one ? reflux_kernel<float, 1> : reflux_kernel<float, 3>, view<float>(*cfg, *forest, *state));
     return e == cudaSuccess ? AF_OK : AF_ERR_CUDA;
 }
 

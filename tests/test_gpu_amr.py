@@ -188,6 +188,37 @@ def test_reflux_matches_oracle(af, prec):
     assert _nerr(d.double().cpu().numpy(), ref_st) < TOL[prec]
 
 
+@pytest.mark.parametrize("n", [2, 6, 20, 64])
+@pytest.mark.parametrize("eq,prec", [(0, 0), (0, 1), (1, 0), (1, 1)])
+def test_reflux_and_planned_fill_of_every_patch_size(af, eq, prec, n):
+    """One and three components, from the smallest patch to the largest, with
+    several levels synchronised: the conservative fix matches the oracle (its
+    correction and the sum are one rounding each) and clears the same
+    registers; the planned exchange equals the direct one bit for bit."""
+    lmax, nc = 3, 1 if eq == 0 else 3
+    tdt = torch.float64 if prec == 0 else torch.float32
+    leaves = _sorted(_diag_forest(2, 3))
+    st = np.nan_to_num(S.random_state(S.Layout(n, nc), len(leaves), seed=n).reshape(len(leaves), -1))
+    st = st.astype(np.float32).astype(np.float64) if prec else st
+    freg = np.random.default_rng(n).uniform(-1, 1, size=(len(leaves), 4 * nc * n))
+    lv, ix, iy = (np.array(v, np.int32) for v in zip(*leaves))
+    ref_st, ref_fr = st.copy(), freg.copy()
+    O.lib().orc_reflux_amr(n, nc, len(leaves), _ip(lv), _ip(ix), _ip(iy), 1, lmax, 0b1110, 0.125, 0.0625,
+                           O._dp(ref_fr), O._dp(ref_st))
+    F = _device_forest(af, leaves, lmax)
+    cfg = af.config(eq, prec, n, 1.0, 0.5, 1.0)
+    d, dfr = torch.from_numpy(st).to(tdt).cuda(), torch.from_numpy(freg).cuda()
+    af.reflux(cfg, F.c, 0b1110, 0.125, 0.0625, dfr, d)
+    assert np.array_equal(dfr.cpu().numpy(), ref_fr)
+    assert _nerr(d.double().cpu().numpy(), ref_st) < (1e-15 if prec == 0 else 2.0 ** -22)
+    plan, n_a, n_b = af.ghost_plan(cfg, F.c)
+    one, two = d.clone(), d.clone()
+    af.fill_ghosts(cfg, F.c, 0b1111, 0b1111, 0, one)
+    af.fill_ghosts_planned(cfg, F.c, 0b1111, 0, plan, n_a, n_b, af.state_pair(two, None, 0))
+    torch.cuda.synchronize()
+    assert n_b > 0 and torch.equal(one, two)
+
+
 @pytest.mark.parametrize("kind", [0, 1])
 def test_tag_and_mass_match_oracle(af, kind):
     n, lmax, nc = 16, 3, 3
