@@ -12,6 +12,8 @@
 
 namespace {
 
+bool ok(cudaError_t e) { return e == cudaSuccess; }
+
 // Events of one call, destroyed on return (the driver keeps what is pending).
 struct Events {
     cudaEvent_t *e = nullptr;
@@ -19,7 +21,7 @@ struct Events {
     explicit Events(int want) {
         e = new (std::nothrow) cudaEvent_t[want];
         if (!e) return;
-        while (n < want && cudaEventCreateWithFlags(&e[n], cudaEventDisableTiming) == cudaSuccess) ++n;
+        while (n < want && ok(cudaEventCreateWithFlags(&e[n], cudaEventDisableTiming))) ++n;
         if (n < want) {
             clear();
         }
@@ -36,8 +38,6 @@ struct Events {
     Events &operator=(const Events &) = delete;
 };
 
-bool ok(cudaError_t e) { return e == cudaSuccess; }
-
 }  // namespace
 
 extern "C" af_status af_step_host_bands(const af_config *cfg, int32_t tiling, int32_t nband, const af_band *h_band,
@@ -50,6 +50,11 @@ extern "C" af_status af_step_host_bands(const af_config *cfg, int32_t tiling, in
     if (cfg->ncomp != (cfg->eq == AF_ADVECTION ? 1 : 3)) return AF_ERR_ARG;
     for (int b = 0; b < nband; ++b)
         if (h_band[b].p0 < 0 || h_band[b].p1 <= h_band[b].p0 || h_band[b].nwork < 0) return AF_ERR_ARG;
+    // a step that would be refused is, before the first copy
+    for (int b = 0; b < nband; ++b) {
+        const af_status st = af::step_check(cfg, tiling, h_band[b].nwork, h_band[b].d_work, d_a, d_b, dt0, dx0, dy0, d_flux_reg);
+        if (st != AF_OK) return st;
+    }
     const size_t esz = cfg->prec == AF_F64 ? 8 : 4;
     const size_t dev = (size_t)af_patch_words(cfg->n, cfg->ncomp) * esz;
     const size_t host = owned ? (size_t)cfg->ncomp * 4 * cfg->n * cfg->n * esz : dev;
@@ -57,7 +62,7 @@ extern "C" af_status af_step_host_bands(const af_config *cfg, int32_t tiling, in
     cudaStream_t cmp = static_cast<cudaStream_t>(s_cmp), out = static_cast<cudaStream_t>(s_out);
     auto at = [](void *base, size_t patch, size_t bytes) { return static_cast<char *>(base) + patch * bytes; };
 
-    Events ev(2 * nband + 3);  // uploaded [nband], stepped [nband], start, end of s_out, end of s_cmp
+    Events ev(2 * nband + 4);  // uploaded [nband], stepped [nband], start, ends of s_out, s_cmp, s_in
     if (ev.n == 0) return AF_ERR_CUDA;
     cudaEvent_t *const up = ev.e, *const done = ev.e + nband, start = ev.e[2 * nband];
     if (!ok(cudaEventRecord(start, cur)) || !ok(cudaStreamWaitEvent(in, start, 0)) ||
@@ -93,10 +98,13 @@ extern "C" af_status af_step_host_bands(const af_config *cfg, int32_t tiling, in
             !ok(cudaMemcpyAsync(at(h_state, p0, host), at(owned ? d_down : d_b, p0, host), bytes, cudaMemcpyDeviceToHost, out)))
             st = AF_ERR_CUDA;
     }
-    // joined even after an error: what was enqueued stays ordered before `stream`
-    const cudaEvent_t end[2] = {ev.e[2 * nband + 1], ev.e[2 * nband + 2]};
-    if (!ok(cudaEventRecord(end[0], out)) || !ok(cudaStreamWaitEvent(cur, end[0], 0)) ||
-        !ok(cudaEventRecord(end[1], cmp)) || !ok(cudaStreamWaitEvent(cur, end[1], 0)))
-        return st == AF_OK ? AF_ERR_CUDA : st;
+    // joined even after an error, by every join that can still be made: what was
+    // enqueued stays ordered before `stream`.  (s_cmp has waited for all uploads
+    // unless a band was left out.)
+    const cudaStream_t last[3] = {out, cmp, in};
+    for (int k = 0; k < (st == AF_OK ? 2 : 3); ++k) {
+        cudaEvent_t end = ev.e[2 * nband + 1 + k];
+        if ((!ok(cudaEventRecord(end, last[k])) || !ok(cudaStreamWaitEvent(cur, end, 0))) && st == AF_OK) st = AF_ERR_CUDA;
+    }
     return st;
 }

@@ -105,6 +105,12 @@ struct AdvectionPairWeights {
     int32_t fold, pad_;
 };
 
+// What af_patch_step_tiled refuses before it launches anything (af_step.cu);
+// AF_OK for an empty work list.
+af_status step_check(const af_config *cfg, int32_t tiling_index, int32_t nwork, const af_work *d_work,
+                     const void *d_in, const void *d_out, double dt0, double dx0, double dy0,
+                     const double *d_flux_reg);
+
 // Double-precision derivations on the host (af_weights.cpp).
 void acoustic_weights(double rho_x, double rho_y, AcousticWeights<double> &w);
 // Folded weights; returns false if the dense weights lack the symmetry

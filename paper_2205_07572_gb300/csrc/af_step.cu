@@ -135,11 +135,10 @@ extern "C" int32_t af_step_default_tiling(const af_config *cfg) {
 }
 
 namespace af {
-namespace {
 
-af_status step_checked(const af_config *cfg, int32_t tiling_index, int32_t nwork, const af_work *d_work,
-                       const void *d_in, void *d_out, uint32_t swap, double dt0, double dx0, double dy0,
-                       double *d_flux_reg, void *stream) {
+af_status step_check(const af_config *cfg, int32_t tiling_index, int32_t nwork, const af_work *d_work,
+                     const void *d_in, const void *d_out, double dt0, double dx0, double dy0,
+                     const double *d_flux_reg) {
     if (cfg == nullptr || nwork < 0) return AF_ERR_ARG;
     if (tiling_index < 0 || tiling_index >= kNumTilings) return AF_ERR_ARG;
     if (cfg->n < 2 || cfg->n > 64) return AF_ERR_ARG;
@@ -162,6 +161,16 @@ af_status step_checked(const af_config *cfg, int32_t tiling_index, int32_t nwork
         if (!(cfg->c > 0.0)) return AF_ERR_ARG;
         if (cfg->c * dt0 / dx0 > 0.5 + tol || cfg->c * dt0 / dy0 > 0.5 + tol) return AF_ERR_CFL;
     }
+    return AF_OK;
+}
+
+namespace {
+
+af_status step_checked(const af_config *cfg, int32_t tiling_index, int32_t nwork, const af_work *d_work,
+                       const void *d_in, void *d_out, uint32_t swap, double dt0, double dx0, double dy0,
+                       double *d_flux_reg, void *stream) {
+    const af_status st = step_check(cfg, tiling_index, nwork, d_work, d_in, d_out, dt0, dx0, dy0, d_flux_reg);
+    if (st != AF_OK || nwork == 0) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int k = tiling_index;
     if (cfg->prec == AF_F64)

@@ -149,12 +149,14 @@ class UniformRun:
                 and host.shape == (self.npatch, words) and host.is_contiguous()):
             return False
         s_in, s_cmp, s_out = self._streams
-        af.step_host_bands(self.cfg, self.tiling, self._bands_c, up is not None, host, up, down, self.a, self.b, self.dt,
-                           self.dx, self.dy, self.freg, None, s_in, s_cmp, s_out)
-        # one element through torch on the caller's stream, which now waits for
-        # every copy of `host`: torch's allocator then knows until when the pinned
-        # block is in use
-        self._mark.copy_(host.view(-1)[:1], non_blocking=True)
+        try:
+            af.step_host_bands(self.cfg, self.tiling, self._bands_c, up is not None, host, up, down, self.a, self.b, self.dt,
+                               self.dx, self.dy, self.freg, None, s_in, s_cmp, s_out)
+        finally:
+            # one element through torch on the caller's stream, which now waits for
+            # every copy of `host` (those of a step that failed part-way too): torch's
+            # allocator then knows until when the pinned block is in use
+            self._mark.copy_(host.view(-1)[:1], non_blocking=True)
         self.t += self.dt
         return True
 

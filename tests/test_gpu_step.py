@@ -676,6 +676,45 @@ def test_host_step_takes_every_form_of_host_state(af, owned, prec, bands, form):
     assert hrun.t == dev.t
 
 
+@pytest.mark.parametrize("owned", [False, True])
+def test_refused_host_step_leaves_the_state_alone(af, owned):
+    """A banded host step beyond the CFL limit raises before anything is copied:
+    the host and device states are as they were, and the steps that follow
+    equal the device's bit for bit."""
+    from paper_2205_07572_gb300.uniform import UniformRun
+    n, px, nc = 8, 16, 3
+    grid = S.UniformGrid(S.Layout(n, nc), px, px)
+    st = S.periodic_state(grid, S.pulse_plus_vortex(), nq=2)
+    cfg = af.config(af.ACOUSTICS, 0, n, c=1.0)
+    dev = UniformRun(cfg, px, px, grid.dx, grid.dy, 0.4 * grid.dx, state=st)
+    hrun = UniformRun(cfg, px, px, grid.dx, grid.dy, 0.4 * grid.dx, state=None)
+    step = hrun.step_host_owned if owned else hrun.step_host
+
+    def host_form():
+        if not owned:
+            return dev.a.cpu()
+        own = torch.empty((grid.npatch, af.owned_words(n, nc)), dtype=dev.a.dtype, device="cuda")
+        af.pack_owned(cfg, grid.npatch, dev.a, own)
+        return own.cpu()
+
+    host = host_form().pin_memory()
+    for _ in range(2):
+        before, a0 = host.clone(), hrun.a.clone()
+        hrun.dt = 0.6 * grid.dx
+        with pytest.raises(af.AFError):
+            step(host, 16)
+        torch.cuda.synchronize()
+        assert torch.equal(host, before) and torch.equal(hrun.a, a0)
+        hrun.dt = dev.dt
+        step(host, 16)
+        dev.step()
+        torch.cuda.synchronize()
+        lay = S.Layout(n, nc)
+        cut = lambda x: x if owned else lay.lattice(x.numpy().reshape(-1, nc, 4, x.shape[1] // (4 * nc)))[..., S.G:S.G + n, S.G:S.G + n]  # noqa: E731
+        assert np.array_equal(cut(host), cut(host_form()))
+    assert hrun.t == dev.t
+
+
 @pytest.mark.parametrize("prec", [0, 1])
 def test_fma_probe_computes_its_chains(af, prec):
     """af_fma_throughput (the ALU-roof probe) runs the chains it claims: every
