@@ -12,7 +12,12 @@
 
 namespace {
 
-bool ok(cudaError_t e) { return e == cudaSuccess; }
+// A failed call's error is reported by the return value, and not once more by
+// whatever call reads the runtime's last error next.
+bool ok(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
+}
 
 // Events of one call, destroyed on return (the driver keeps what is pending).
 struct Events {

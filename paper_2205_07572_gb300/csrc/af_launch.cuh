@@ -46,7 +46,10 @@ inline cudaError_t launch_chained(bool chain, void (*kern)(P...), dim3 grid, dim
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, P(std::forward<Args>(args))...);
+    // reported here, and not once more by whatever call reads the last error next
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P(std::forward<Args>(args))...);
+    const cudaError_t last = cudaGetLastError();
+    return e != cudaSuccess ? e : last;
 }
 
 }  // namespace af

@@ -128,3 +128,37 @@ def test_every_enqueued_operation_is_ordered_before_the_callers_stream(model, nb
 def test_a_refused_step_copies_nothing(model, owned):
     st, copies, ops, covered, pending, events = model(5, owned, dt=2.0)
     assert st != 0 and copies == 0 and ops == 0
+
+
+@pytest.mark.parametrize("kind", [1, 2, 3])
+def test_no_runtime_error_is_left_pending(model, kind):
+    """The failed call's error is returned, and the call that reads the
+    runtime's last error next does not see it again."""
+    for at in range(1, 5):  # two bands: four copies, at least as many event operations
+        st, _, _, _, pending, _ = model(2, 1, kind, at)
+        assert st != 0 and pending == 0, (kind, at)
+
+
+@pytest.mark.gpu
+def test_a_refused_launch_is_reported_once(tmp_path):
+    """launch_chained returns a launch's error (1 MB of shared memory: refused
+    by the host; nothing runs) and does not leave it to the next call that reads
+    the last error.  (A machine without a driver reports that at every call.)"""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("needs nvcc")
+    (tmp_path / "launch.cu").write_text(r"""
+#include <cstdio>
+#include "af_launch.cuh"
+__global__ void kern(int *out) { *out = (int)af::chain_begin(); }
+int main() {
+    const cudaError_t e = af::launch_chained(true, kern, 1, 32, 1 << 20, nullptr, (int *)nullptr);
+    printf("%d %d\n", (int)e, (int)cudaPeekAtLastError());
+    return 0;
+}
+""")
+    exe = str(tmp_path / "launch")
+    subprocess.run([nvcc, "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-I",
+                    os.path.join(ROOT, "paper_2205_07572_gb300", "csrc"), str(tmp_path / "launch.cu"), "-o", exe], check=True)
+    e, pending = (int(v) for v in subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split())
+    assert e != 0 and pending == 0
