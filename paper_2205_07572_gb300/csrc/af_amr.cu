@@ -1187,8 +1187,11 @@ extern "C" af_status af_ghost_plan_build(const af_config *cfg, const af_forest *
     // scratch: two slot cursors and an overflow flag
     if (cudaMemsetAsync(d_scratch, 0, 3 * sizeof(int64_t), s) != cudaSuccess) return AF_ERR_CUDA;
     if (forest->nleaf == 0) return AF_OK;
-    const size_t held = (size_t)kPlanes * ring_count(cfg->n) * sizeof(GhostEntry);  // up to 52 KB (n = 64)
-    if (cudaFuncSetAttribute(plan_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)held) != cudaSuccess)
+    const size_t held = (size_t)kPlanes * ring_count(cfg->n) * sizeof(GhostEntry);
+    // the limit of the largest patches (51 KB), whatever this call's: it belongs to
+    // the kernel, and another thread may be about to launch it for larger patches
+    constexpr int limit = kPlanes * ring_count(64) * (int)sizeof(GhostEntry);
+    if (cudaFuncSetAttribute(plan_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess)
         return AF_ERR_CUDA;
     plan_build_kernel<<<forest->nleaf, 256, held, s>>>(
         make_dev(*forest, cfg->n), plane_stride(cfg->n), flags, static_cast<GhostEntry *>(d_plan), n_a, n_b,

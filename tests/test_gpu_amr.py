@@ -219,6 +219,41 @@ def test_reflux_and_planned_fill_of_every_patch_size(af, eq, prec, n):
     assert n_b > 0 and torch.equal(one, two)
 
 
+def test_plans_of_different_patch_sizes_from_two_threads(af):
+    """Two host threads build the ghost plans of the largest and of small patches
+    at the same time, on streams of their own: every call succeeds and finds the
+    entries that a single thread finds."""
+    import threading
+    lmax = 3
+    leaves = _sorted(_diag_forest(2, 3))
+    F = _device_forest(af, leaves, lmax)
+    cfgs = [af.config(0, 1, n) for n in (64, 4)]
+    entries = lambda p: torch.sort(p.view(-1, af.GHOST_ENTRY_BYTES // 8), dim=0)[0]  # noqa: E731
+    ref = [af.ghost_plan(c, F.c) for c in cfgs]
+    ref = [(entries(p), n_a, n_b) for p, n_a, n_b in ref]
+    torch.cuda.synchronize()
+    failed = []
+    gate = threading.Barrier(2)
+
+    def build(k):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                gate.wait()
+                for _ in range(1500):
+                    plan, n_a, n_b = af.ghost_plan(cfgs[k], F.c)
+                    assert (n_a, n_b) == ref[k][1:]
+                assert torch.equal(entries(plan), ref[k][0])
+        except Exception as e:  # noqa: BLE001
+            failed.append((k, repr(e)))
+
+    threads = [threading.Thread(target=build, args=(k,)) for k in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
+
+
 @pytest.mark.parametrize("kind", [0, 1])
 def test_tag_and_mass_match_oracle(af, kind):
     n, lmax, nc = 16, 3, 3
