@@ -141,13 +141,18 @@ class UniformRun:
 
     def _step_host_native(self, host, words: int, up, down) -> bool:
         """The banded step enqueued by one native call, if `host` is what that
-        takes: a CPU tensor of the state's type and exactly its shape, dense.
-        Anything else (another type, strides, broadcasting) goes through
-        torch's copies."""
+        takes: a plain CPU tensor of the state's type and exactly its shape,
+        dense.  Anything else (another type, strides, broadcasting, a subclass,
+        a lazily negated tensor) goes through torch's copies, and so does what
+        those refuse to write to: a tensor that requires a gradient, or one made
+        in inference mode outside of it."""
         import torch
-        if not (isinstance(host, torch.Tensor) and host.device.type == "cpu" and host.dtype == self.a.dtype
-                and host.shape == (self.npatch, words) and host.is_contiguous()):
+        if not (type(host) in (torch.Tensor, torch.nn.Parameter) and host.device.type == "cpu" and host.dtype == self.a.dtype
+                and host.shape == (self.npatch, words) and host.is_contiguous() and not host.requires_grad
+                and not host.is_neg() and (not host.is_inference() or torch.is_inference_mode_enabled())):
             return False
+        if not host.is_inference():
+            torch.autograd.graph.increment_version(host)  # written in place, as by copy_
         s_in, s_cmp, s_out = self._streams
         try:
             af.step_host_bands(self.cfg, self.tiling, self._bands_c, up is not None, host, up, down, self.a, self.b, self.dt,
