@@ -918,8 +918,8 @@ __global__ void reflux_kernel(const __grid_constant__ DevForest F, StateView<T> 
     const int64_t total = (int64_t)F.nleaf * 4 * n;
     const unsigned block = chain_begin();
     for (int64_t t = block * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        // 32-bit divisions (total < 2^31 for any state that fits the GPU)
-        const int f = (int)t / n, k = (int)t - f * n, p = f >> 2, side = f & 3;
+        int p, side, k;
+        face_entry(t, n, p, side, k);
         const int l = __ldg(F.level + p);
         if (l >= AF_MAX_LEVEL || !((sync >> l) & 1u) || !((sync >> (l + 1)) & 1u)) continue;
         const int hw = hwid(F, l), x0 = leaf_x0(F, p), y0 = leaf_y0(F, p);

@@ -39,6 +39,17 @@ AF_HD constexpr int64_t plane_stride(int n) {
     return ((int64_t)(n + 2 * kGhost + 1) * (n + 2 * kGhost + 1) + 7) / 8 * 8;
 }
 
+// Flux-register entry t of a forest of patches of n cells: cell k along a side
+// of patch p.  Unsigned 32-bit divisions: fewer than 2^32 entries of any state
+// that fits the GPU (patches of two cells take over 900 bytes each with their
+// registers, and have eight entries), but more than 2^31 may.
+AF_HD inline void face_entry(int64_t t, int n, int &p, int &side, int &k) {
+    const uint32_t f = (uint32_t)t / (uint32_t)n;
+    k = (int)((uint32_t)t - f * (uint32_t)n);
+    p = (int)(f >> 2);
+    side = (int)(f & 3u);
+}
+
 AF_HD constexpr int x_idx(int k) {
     constexpr int t[15] = {2, 3, 7, 8, 9, 10, 11, 12, 16, 17, 18, 21, 22, 23, 24};
     return t[k];
