@@ -89,7 +89,6 @@ __device__ __forceinline__ void cp_async(double *smem, const double *gmem) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
 // Issue (without waiting) the copies of the window of node lines
 // [x0-1, x1+1] x [y0-1, y1+1] of every plane of work item wk into Sin
@@ -1022,29 +1021,6 @@ __device__ __forceinline__ bool stage_bulk_ext(const StepArgs<T> &A, const af_wo
     return true;
 }
 
-// Issue (every thread, without waiting) the halo copies of a bulk-staged
-// tile whose bulk copies have landed.
-template <typename T, int NT, int WX, int WSZ, int NC>
-__device__ __forceinline__ void halo_async(const StepArgs<T> &A, const af_work &wk, T *Sin) {
-    constexpr int n = WX - 2 * kGhost - 1;
-    constexpr int ncp = NC * kPlanes;
-    constexpr int64_t plane = plane_stride(n), pw = ncp * plane;
-    const T *const in = src_buf(A, wk.level);
-    int nb[8];
-#pragma unroll
-    for (int d = 0; d < 8; ++d) nb[d] = wk.nbr[d];
-    const HaloList<n> H(wk.y0, wk.y1);
-    for (int t = threadIdx.x; t < H.count; t += NT) {
-        int li, lj, so;
-        const int q = H.entry(nb, t, li, lj, so);
-        if (q < 0) continue;
-        const T *g = in + (int64_t)q * pw + so;
-        T *sp = Sin + (lj - H.y0 + 1) * WX + (li + 1);
-#pragma unroll
-        for (int cp = 0; cp < ncp; ++cp) cp_async(sp + cp * WSZ, g + cp * plane);
-    }
-}
-
 // For a bulk-staged tile: write the ghost columns (-2, -1, n, n+1, n+2) of
 // the lattice rows y0 .. y1-1 the tile writes, in every plane, with the
 // staged t^n values.  The tile's rows then go out whole, so consecutive rows
@@ -1069,10 +1045,6 @@ __device__ __forceinline__ void write_ghost_columns(const StepArgs<T> &A, const 
         for (int cp = 0; cp < ncp; ++cp) __stcs(o + cp * plane, sp[cp * WSZ]);
     }
 }
-
-// Order this thread's generic-proxy accesses to shared memory before later
-// bulk (async-proxy) writes to the same buffer.
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
 // One tile per CTA.  SPLIT: gridDim.y CTAs share a tile, each a band of its
 // rows, as if the tile had been built that way (few_tiles).
@@ -1127,119 +1099,6 @@ __global__ void __launch_bounds__(NT, (min_ctas<T, EQ, NT>())) step_kernel(const
     if (bulk_tile<T, Gm::WX>(A, wk)) write_ghost_columns<T, NT, Gm::WX, Gm::WSZ, ncomp>(A, wk, Sin);
 }
 
-// How a persistent CTA stages a work item: 0 not at all (built for another
-// tiling), 1 element by element, 2 in bulk.
-template <typename T, int WX, int TMX, int TMY>
-__device__ __forceinline__ int stage_kind(const StepArgs<T> &A, const af_work &w) {
-    if (w.x1 - w.x0 > TMX || w.y1 - w.y0 > TMY) return 0;
-    return bulk_tile<T, WX>(A, w) ? 2 : 1;
-}
-
-// Persistent variant (not launched: launch_tiling refuses persistent
-// tilings): one CTA loops over work items t, t + gridDim.x, ...
-// with two windows, so staging overlaps compute.  The copies of the next
-// tile are issued before the node phase of the current one: its bulk copies
-// (thread 0), or its element-wise copies.  A bulk-staged next tile's halo
-// copies follow between the current tile's node and flux phases, once its
-// bulk copies have landed.  A wait that gives up ends the CTA (its remaining
-// tiles stay unwritten) after counting it in g_wait_timeouts.
-template <typename T, int EQ, int NT, int TMX, int TMY, int NN = 0>
-__global__ void __launch_bounds__(NT, (min_ctas<T, EQ, NT>())) step_kernel_pipe(const __grid_constant__ StepArgs<T> A,
-                                                       const __grid_constant__ typename WeightsOf<T, EQ>::type W,
-                                                       int nwork) {
-    using Gm = Geo<TMX, TMY, NN>;
-    constexpr int ncomp = (EQ == AF_ACOUSTICS) ? 3 : 1;
-    constexpr int wbuf = ncomp * kPlanes * Gm::WSZ;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *const S0 = reinterpret_cast<T *>(smem_raw) + win_off<T, Gm::WX>();
-    T *const ST = reinterpret_cast<T *>(smem_raw) + 2 * wbuf;
-    __shared__ __align__(8) uint64_t bar[2];
-    int t = blockIdx.x;
-    if (t >= nwork) return;
-    if (threadIdx.x == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-    }
-    __syncthreads();
-    unsigned phase = 0;  // bit b: parity of the next phase of bar[b]
-    bool ok = true;
-    {  // the first tile, staged completely
-        const int kind = stage_kind<T, Gm::WX, TMX, TMY>(A, A.work[t]);
-        if (kind == 2) {
-            if (threadIdx.x == 0) bulk_issue<T, Gm::WX, Gm::WSZ, ncomp>(A, A.work[t], S0, &bar[0]);
-            ok = mbar_wait(&bar[0], 0);
-            phase = 1;
-            halo_async<T, NT, Gm::WX, Gm::WSZ, ncomp>(A, A.work[t], S0);
-        } else if (kind == 1) {
-            stage_issue<T, NT, Gm::WX, Gm::WSZ, ncomp, NN>(A, A.work[t], S0);
-        }
-        cp_async_commit();
-        cp_async_wait_all();
-        if (__syncthreads_or(!ok)) {
-            if (threadIdx.x == 0) {
-                atomicAdd(&g_wait_timeouts, 1u);
-                mbar_wait(&bar[0], 0);
-            }
-            return;
-        }
-    }
-    int b = 0;
-    for (; t < nwork; t += gridDim.x) {
-        const int tn = t + gridDim.x;
-        T *const Sc = S0 + b * wbuf;
-        T *const Sn = S0 + (b ^ 1) * wbuf;
-        int nkind = 0;
-        if (tn < nwork) {
-            nkind = stage_kind<T, Gm::WX, TMX, TMY>(A, A.work[tn]);
-            if (nkind == 2) {
-                if (threadIdx.x == 0) bulk_issue<T, Gm::WX, Gm::WSZ, ncomp>(A, A.work[tn], Sn, &bar[b ^ 1]);
-            } else if (nkind == 1) {
-                stage_issue<T, NT, Gm::WX, Gm::WSZ, ncomp, NN>(A, A.work[tn], Sn);
-                cp_async_commit();
-            }
-        }
-        const af_work wk = A.work[t];
-        const bool fits = wk.x1 - wk.x0 <= TMX && wk.y1 - wk.y0 <= TMY;
-        if (fits) {
-            if (wk.flags & 1) {
-                stage_copy_out<T, NT, Gm::WX, Gm::WSZ, ncomp, NN>(A, wk, Sc);
-                __syncthreads();  // copies land before the computed values overwrite them
-            }
-            tile_nodes<T, EQ, NT, Gm::WX, Gm::WSZ, Gm::TX, Gm::TSZ, TMX, NN>(A, W, Sc, ST, wk.patch, wk.level,
-                                                                            wk.x0, wk.x1, wk.y0, wk.y1);
-        }
-        __syncthreads();
-        unsigned par = 0;
-        if (nkind == 2) {
-            par = (phase >> (b ^ 1)) & 1u;
-            ok = mbar_wait(&bar[b ^ 1], par);
-            phase ^= 1u << (b ^ 1);
-            halo_async<T, NT, Gm::WX, Gm::WSZ, ncomp>(A, A.work[tn], Sn);
-            cp_async_commit();
-        }
-        if (fits) {
-            tile_fluxes<T, EQ, NT, Gm::WX, Gm::WSZ, Gm::TX, Gm::TSZ, TMX, NN, true>(A, Sc, ST, wk.patch, wk.level, wk.x0, wk.x1,
-                                                                              wk.y0, wk.y1);
-            if (A.freg != nullptr) {
-                BoundaryFluxes<T, EQ, NT, Gm::TX, Gm::TSZ, NN> B;
-                B.begin(A, ST, wk.patch, wk.x0, wk.x1, wk.y0, wk.y1);
-                B.end(A, ST, wk.patch, wk.level, wk.x0, wk.x1, wk.y0, wk.y1);
-            }
-            if (bulk_tile<T, Gm::WX>(A, wk)) write_ghost_columns<T, NT, Gm::WX, Gm::WSZ, ncomp>(A, wk, Sc);
-        }
-        cp_async_wait_all();
-        fence_proxy_async();  // this window is refilled by bulk copies after the barrier
-        if (__syncthreads_or(!ok)) {
-            if (threadIdx.x == 0) {
-                atomicAdd(&g_wait_timeouts, 1u);
-                mbar_wait(&bar[b ^ 1], par);  // bounded: the copies in flight
-            }
-            return;
-        }
-        b ^= 1;
-    }
-}
-
 }  // namespace dev
 
 template <typename Kern>
@@ -1267,10 +1126,9 @@ af_status launch_tiling(const StepArgs<T> &A, const typename WeightsOf<T, EQ>::t
     const size_t win = sizeof(T) * (size_t)ncomp * kPlanes * Gm::WSZ;
     const size_t tarr = sizeof(T) * (size_t)ncomp * 3 * Gm::TSZ;
     if constexpr (PIPE) {
-        // The persistent (two-window) kernel is not launched: in two
-        // experimental builds a launch of it on 48 x 48 patches ended in an
-        // unspecified launch failure, and reading its schedule has not found
-        // the cause.  Until it is found, persistent tilings are refused.
+        // There is no persistent (two-window) kernel: in two experimental
+        // builds a launch of it on 48 x 48 patches ended in an unspecified
+        // launch failure whose cause was not found, and it was the slower one.
         (void)win;
         (void)tarr;
         return AF_ERR_UNIMPLEMENTED;
