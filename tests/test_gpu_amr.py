@@ -254,6 +254,36 @@ def test_plans_of_different_patch_sizes_from_two_threads(af):
     assert not failed, failed
 
 
+@pytest.mark.parametrize("n", [2, 7, 16, 33])
+@pytest.mark.parametrize("kind", [0, 1])
+def test_indicator_is_exact(af, kind, n):
+    """Only maxima, one subtraction and one division form an indicator, so it
+    equals numpy's bit for bit: on every level, with mesh widths that are no
+    powers of two, missing values ignored, infinite ones kept."""
+    lmax, nc, dx, dy = 3, 3, 0.3, 0.7
+    leaves = _sorted(_diag_forest(1, 3))
+    lay = S.Layout(n, nc)
+    st = S.random_state(lay, len(leaves), seed=n + kind)
+    q = np.nan_to_num(lay.lattice(st)[:, 1, 0, G:G + n, G:G + n])
+    q[0], q[2, 0, 0], q[3, n - 1, n // 2], q[4] = 0.0, np.nan, np.inf, -1.5
+    lay.lattice(st)[:, 1, 0, G:G + n, G:G + n] = q
+    F = _device_forest(af, leaves, lmax)
+    d = torch.from_numpy(st.reshape(len(leaves), -1)).cuda()
+    t, ind = torch.zeros(len(leaves), dtype=torch.int8, device="cuda"), torch.zeros(len(leaves), dtype=torch.float64, device="cuda")
+    af.tag(af.config(1, 0, n, c=1.0), F.c, d, 1, kind, dx, dy, 0.9, 0.2, t, ind)
+    torch.cuda.synchronize()
+    h = 0.5 ** np.array([l for l, _, _ in leaves])[:, None, None]
+    with np.errstate(invalid="ignore"):
+        if kind == 0:
+            ref = np.nanmax(q, axis=(1, 2)) - np.nanmin(q, axis=(1, 2))
+        else:
+            gx = np.abs(q[:, 1:-1, 2:] - q[:, 1:-1, :-2]) / (2.0 * (dx * h))
+            gy = np.abs(q[:, 2:, 1:-1] - q[:, :-2, 1:-1]) / (2.0 * (dy * h))
+            ref = np.fmax(np.fmax.reduce(np.fmax(gx, gy).reshape(len(leaves), -1), axis=1, initial=-np.inf), 0.0)
+    assert np.array_equal(ind.cpu().numpy(), ref)
+    assert np.array_equal(t.cpu().numpy(), np.where(ref >= 0.9, 1, np.where(ref < 0.2, -1, 0)))
+
+
 @pytest.mark.parametrize("kind", [0, 1])
 def test_tag_and_mass_match_oracle(af, kind):
     n, lmax, nc = 16, 3, 3
