@@ -151,6 +151,46 @@ AF_HD constexpr Tiling tiling(int k) {
 // the autotuner through the *_tiled entry points).
 inline int default_tiling(int n) { return n <= 8 ? 8 : (n <= 16 ? 6 : 0); }
 
+constexpr int kSMs = 152;
+
+// CTAs that share each of `nwork` tiles, as bands of its rows (step_kernel,
+// SPLIT): one, two on an SM at most, or as many as give every SM one, whichever
+// the following estimate of the fullest SM's time finds cheapest.  A band costs
+// the warps of its nodes -- a row more than its cells' -- on the SM it shares
+// with others, and the turns its threads take over them cost latency; two bands
+// on an SM hide each other's waits in FP32 and stand in one queue for the FP64
+// pipe; and FP32 kernels compiled for a patch size (launch_step) have cheaper
+// rows than the ones that split, those that stage a whole lattice in bulk by
+// far.  The constants are fitted to every tiling at 8 to 32 cells and 1 to 152
+// tiles: within 5 % of the better of whole tiles and two bands an SM nearly
+// everywhere (7 % at worst), up to 7x faster than whole tiles.  (Two bands an
+// SM always: 102 to 152 tiles of 32 x 32 FP64 cells took 156 us for 140
+// acoustics, 35.7 for 24.7 advection.)  One 64 x 64 FP64 patch in 32 x 32 tiles:
+// 24.7 us a step on four CTAs, 5.5 on 64.
+// adaptive: the patches mostly advance their first ghost layer too.
+inline int few_tiles(bool f64, bool acoustics, const Tiling &t, int nwork, int n, bool adaptive) {
+    if (nwork < 1 || nwork > kSMs) return 1;
+    auto up = [](int a, int b) { return (a + b - 1) / b; };
+    const int w = adaptive ? n + 2 : n;
+    const int tw = up(w, up(w, t.tmx)), th = up(w, up(w, t.tmy));  // a tile (near-equal parts)
+    const bool compiled = !f64 && (n == 16 || n == 32), lattice = t.tmx == n + 2 && t.tmy == n + 2;
+    const double turn = acoustics ? 4.0 : (f64 ? 8.0 : 6.0);
+    const double shared = f64 ? 1.25 : (acoustics ? 1.1 : 0.8);
+    const double generic = !compiled ? 1.0 : (!acoustics || lattice ? 1.3 : 1.05);
+    auto cost = [&](int s) {
+        const int bands = up(nwork * s, kSMs), nodes = (tw + 1) * (up(th, s) + 1);
+        return (bands * up(nodes, 32) + turn * up(nodes, t.threads)) * (bands > 1 ? shared : 1.0) * (s > 1 ? generic : 1.0);
+    };
+    const int rows = n + 2 < t.tmy ? n + 2 : t.tmy, most = rows / 2 < 1 ? 1 : rows / 2;  // bands of two rows or more
+    int best = 1;
+    for (int per = 1; per <= 2; ++per) {
+        const int s = per * kSMs / nwork;
+        const int c = s < most ? s : most;
+        if (cost(c) < cost(best)) best = c;
+    }
+    return best;
+}
+
 // Split `w` cells into ceil(w / kTileMax) tiles of near-equal size.
 inline int tiles_for(int w) { return (w + kTileMax - 1) / kTileMax; }
 inline int tile_size_max(int w) {

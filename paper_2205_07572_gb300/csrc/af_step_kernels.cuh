@@ -1107,17 +1107,6 @@ inline cudaError_t ensure_smem(Kern k, size_t bytes) {
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-// CTAs that share each of `nwork` tiles of up to `rows` rows (step_kernel,
-// SPLIT): one, unless the tiles leave most of the GPU's 152 SMs idle.  Then as
-// many as bring two CTAs to an SM, of two rows or more: a band's extra row of
-// nodes costs up to half its work again, on SMs that would do nothing.  One
-// 64 x 64 FP64 patch in 32 x 32 tiles: 28.7 us on four CTAs, 9.2 us on 64,
-// where the host's share of a call set the time (5.2 us since that shrank).
-inline int few_tiles(int nwork, int rows) {
-    const int s = 2 * 152 / (nwork < 1 ? 1 : nwork), most = rows / 2;
-    return s < 2 ? 1 : (s < most ? s : (most < 1 ? 1 : most));
-}
-
 template <typename T, int EQ, int NT, int TMX, int TMY, int PIPE, int NN>
 af_status launch_tiling(const StepArgs<T> &A, const typename WeightsOf<T, EQ>::type &W, int nwork,
                         cudaStream_t stream) {
@@ -1138,7 +1127,7 @@ af_status launch_tiling(const StepArgs<T> &A, const typename WeightsOf<T, EQ>::t
         const size_t smem = win + tarr;
         if (smem > 227 * 1024) return AF_ERR_UNIMPLEMENTED;
         if constexpr (NN == 0) {
-            const int split = few_tiles(nwork, A.n + 2 < TMY ? A.n + 2 : TMY);
+            const int split = few_tiles(sizeof(T) == 8, EQ == AF_ACOUSTICS, {TMX, TMY, NT, 0}, nwork, A.n, A.freg != nullptr);
             if (split > 1) {
                 auto kern = dev::step_kernel<T, EQ, NT, TMX, TMY, 0, true>;
                 if (ensure_smem(kern, smem) != cudaSuccess) return AF_ERR_CUDA;
@@ -1199,7 +1188,7 @@ template <typename T, int EQ>
 af_status launch_step(int k, const StepArgs<T> &A, const typename WeightsOf<T, EQ>::type &W, int nwork,
                       cudaStream_t stream) {
     // (few tiles are split further, by the kernels for any size)
-    if constexpr (sizeof(T) == 4) if (few_tiles(nwork, 4) == 1) {
+    if constexpr (sizeof(T) == 4) if (few_tiles(false, EQ == AF_ACOUSTICS, tiling(k), nwork, A.n, A.freg != nullptr) == 1) {
         if (A.n == 16) return launch_step_nn<T, EQ, 16>(k, A, W, nwork, stream);
         if (A.n == 32) return launch_step_nn<T, EQ, 32>(k, A, W, nwork, stream);
     }
