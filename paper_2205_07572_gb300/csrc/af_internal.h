@@ -155,7 +155,8 @@ constexpr int kSMs = 152;
 
 // CTAs that share each of `nwork` tiles, as bands of its rows (step_kernel,
 // SPLIT): one, two on an SM at most, or as many as give every SM one, whichever
-// the following estimate of the fullest SM's time finds cheapest.  A band costs
+// the following estimate of the fullest SM's time finds cheapest (whole tiles
+// unless bands are 3 % cheaper).  A band costs
 // the warps of its nodes -- a row more than its cells' -- on the SM it shares
 // with others, and the turns its threads take over them cost latency; two bands
 // on an SM hide each other's waits in FP32 and stand in one queue for the FP64
@@ -186,7 +187,7 @@ inline int few_tiles(bool f64, bool acoustics, const Tiling &t, int nwork, int n
     for (int per = 1; per <= 2; ++per) {
         const int s = per * kSMs / nwork;
         const int c = s < most ? s : most;
-        if (cost(c) < cost(best)) best = c;
+        if (cost(c) < (best == 1 ? 0.97 : 1.0) * cost(best)) best = c;
     }
     return best;
 }
