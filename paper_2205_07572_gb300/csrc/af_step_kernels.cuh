@@ -28,6 +28,8 @@
 
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "af_internal.h"
 #include "af_launch.cuh"
 
@@ -1107,6 +1109,30 @@ inline cudaError_t ensure_smem(Kern k, size_t bytes) {
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// Launch of a step kernel, chained to the one before it (launch_chained) unless
+// that unbalances the SMs (chain_even).  FP32 steps, which take 4 to 15 us where
+// it does, are shorter chained all the same where a stream's launch gap counts
+// (0.65 to 1.12 of the unchained time, mostly below 1); two large tiles an SM
+// gain nothing from it in a graph (256 tiles of 32 x 32 cells 13.6 us, 14.5
+// chained).  FP64 advection of an adaptive run: chain_even_mixed (coarse step of
+// 1144 leaves of 8 x 8 cells 103 us, 126 all chained).
+template <auto Kern, int NT, typename T, typename Wt>
+af_status launch_tiles(const StepArgs<T> &A, const Wt &W, int nwork, int split, size_t smem, cudaStream_t stream) {
+    constexpr bool f64 = sizeof(T) == 8, acoustics = !std::is_same<Wt, AdvectionPairWeights<T>>::value;
+    if (ensure_smem(Kern, smem) != cudaSuccess) return AF_ERR_CUDA;
+    bool chain = !(f64 && acoustics);
+    const int64_t grid = (int64_t)nwork * split;
+    if (chain && grid > kSMs) {
+        const int r = resident_ctas<Kern>(NT, smem);
+        const bool even = chain_even(grid, r);
+        if (f64)
+            chain = A.freg == nullptr ? even : chain_even_mixed(grid, r);
+        else if (!even || r <= 2)
+            chain = !recording(stream);
+    }
+    return launch_chained(chain, Kern, dim3(nwork, split), NT, smem, stream, A, W) == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+}
+
 template <typename T, int EQ, int NT, int TMX, int TMY, int PIPE, int NN>
 af_status launch_tiling(const StepArgs<T> &A, const typename WeightsOf<T, EQ>::type &W, int nwork,
                         cudaStream_t stream) {
@@ -1122,22 +1148,14 @@ af_status launch_tiling(const StepArgs<T> &A, const typename WeightsOf<T, EQ>::t
         (void)tarr;
         return AF_ERR_UNIMPLEMENTED;
     } else {
-        constexpr bool chain = sizeof(T) == 4 || EQ == AF_ADVECTION;
         // (8 TSZ words are used of the 9 where the T arrays are packed)
         const size_t smem = win + tarr;
         if (smem > 227 * 1024) return AF_ERR_UNIMPLEMENTED;
         if constexpr (NN == 0) {
             const int split = few_tiles(sizeof(T) == 8, EQ == AF_ACOUSTICS, {TMX, TMY, NT, 0}, nwork, A.n, A.freg != nullptr);
-            if (split > 1) {
-                auto kern = dev::step_kernel<T, EQ, NT, TMX, TMY, 0, true>;
-                if (ensure_smem(kern, smem) != cudaSuccess) return AF_ERR_CUDA;
-                return launch_chained(chain, kern, dim3(nwork, split), NT, smem, stream, A, W) == cudaSuccess ? AF_OK
-                                                                                                     : AF_ERR_CUDA;
-            }
+            if (split > 1) return launch_tiles<dev::step_kernel<T, EQ, NT, TMX, TMY, 0, true>, NT>(A, W, nwork, split, smem, stream);
         }
-        auto kern = dev::step_kernel<T, EQ, NT, TMX, TMY, NN>;
-        if (ensure_smem(kern, smem) != cudaSuccess) return AF_ERR_CUDA;
-        return launch_chained(chain, kern, nwork, NT, smem, stream, A, W) == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+        return launch_tiles<dev::step_kernel<T, EQ, NT, TMX, TMY, NN>, NT>(A, W, nwork, 1, smem, stream);
     }
 }
 

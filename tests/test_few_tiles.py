@@ -1,4 +1,5 @@
-"""CPU check of the rule that shares few tiles among the idle SMs."""
+"""CPU checks of the rules that decide how a step is launched: few tiles shared
+among the idle SMs, and which grids are chained."""
 import os
 import shutil
 import subprocess
@@ -54,3 +55,27 @@ def test_tiles_that_bands_would_only_slow_down_stay_whole(few):
         assert few(args) == [1] * len(args), args
     # one 64 x 64 patch is four tiles: bands of two rows
     assert few([(1, 0, 0, 4, 64, 0)]) == [16]
+
+
+def test_grids_that_a_chain_would_pile_up_are_not_chained(tmp_path):
+    """(CTAs, resident CTAs an SM) that measured 10 to 50 % slower chained, and
+    neighbours on either side that did not."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("needs nvcc")
+    (tmp_path / "c.cu").write_text(r"""
+#include <cstdio>
+#include <cstdlib>
+#include "af_launch.cuh"
+int main(int argc, char **argv) {
+    for (int i = 1; i + 1 < argc; i += 2) printf("%d\n", (int)af::chain_even(atoll(argv[i]), atoi(argv[i + 1])));
+}
+""")
+    exe = str(tmp_path / "c")
+    subprocess.run([nvcc, "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I",
+                    os.path.join(ROOT, "paper_2205_07572_gb300", "csrc"), str(tmp_path / "c.cu"), "-o", exe], check=True)
+    uneven = [(240, 3), (280, 3), (310, 4), (400, 4), (400, 5), (560, 5), (500, 6), (700, 6), (650, 8), (1000, 8), (760, 9)]
+    even = [(1, 1), (152, 3), (228, 3), (310, 3), (304, 4), (500, 4), (350, 5), (650, 5), (456, 6), (800, 6), (608, 8),
+            (1216, 8), (650, 9), (1, 2), (3000, 1), (10 ** 6, 12)]
+    out = subprocess.run([exe] + [str(v) for e in uneven + even for v in e], check=True, capture_output=True, text=True)
+    assert [int(v) for v in out.stdout.split()] == [0] * len(uneven) + [1] * len(even)

@@ -158,7 +158,7 @@ int main() {
 }
 """)
     exe = str(tmp_path / "launch")
-    subprocess.run([nvcc, "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-I",
+    subprocess.run([nvcc, "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-I", os.path.join(ROOT, "include"), "-I",
                     os.path.join(ROOT, "paper_2205_07572_gb300", "csrc"), str(tmp_path / "launch.cu"), "-o", exe], check=True)
     e, pending = (int(v) for v in subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split())
     assert e != 0 and pending == 0
