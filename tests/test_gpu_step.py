@@ -827,3 +827,137 @@ def test_whole_patch_bulk_staging_equals_elementwise_staging(af, neighbours):
         outs.append(dout.cpu().numpy())
     assert np.array_equal(outs[0], outs[1])
     assert af.step_wait_timeouts() == 0
+
+
+# Launches of up to 152 tiles may be cut into row bands, by kernels for any patch
+# size; 13 x 13 patches run the kernels of large grids in every tiling.
+MANY = 13
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("eq", [0, 1])
+@pytest.mark.parametrize("n", [8, 16, 23, 32])
+@pytest.mark.parametrize("ghosts", ["neighbours", "own"])
+def test_many_tiles_match_oracle_and_equal_few(af, ghosts, n, eq, prec):
+    """Every tiling on more than 152 tiles, with flux registers and without,
+    patches that read their neighbours or their own ghost rings: sampled patches
+    and their registers (every face, component and entry) equal the oracle's, and
+    the same tiles launched a few at a time give the same bits."""
+    nc, P = 1 if eq == 0 else 3, MANY * MANY
+    grid = S.UniformGrid(S.Layout(n, nc), MANY, MANY)
+    own = S.random_owned(grid, seed=5 * n + eq)
+    if prec:
+        own = own.astype(np.float32).astype(np.float64)
+    st = _pack_periodic(grid, own)
+    a, b, c, cfg = 0.9, -0.4, 1.0, af.config(eq, prec, n, 0.9, -0.4, 1.0)
+    dt = _dt(eq, 0.45, grid.dx, grid.dy, a, b, c)
+    cf = O.cfg(eq, n, grid.dx, grid.dy, dt, a, b, c)
+    sample = [0, 1, 7 * MANY + 3, 8 * MANY - 1, P - 1]
+    ref, fref = [], []
+    for p in sample:
+        fr = np.zeros(4 * nc * n)
+        ref.append(O.step_patch(cf, st[p], fr))
+        fref.append(fr.reshape(4, nc, n))
+    ref, fref = np.stack(ref), np.stack(fref)
+    assert (np.abs(fref) > 0).any(axis=(0, 3)).sum() == (4 if eq == 0 else 8)
+    lay = S.Layout(n, nc)
+    cut = lambda x: lay.lattice(x.reshape(-1, nc, 4, x.size // len(x) // (4 * nc)))[..., S.G:S.G + n, S.G:S.G + n]  # noqa: E731
+    tdt = torch.float64 if prec == 0 else torch.float32
+    from paper_2205_07572_gb300.uniform import periodic_neighbours
+    nbr = periodic_neighbours(MANY, MANY) if ghosts == "neighbours" else None
+    din = torch.from_numpy(st.reshape(P, -1)).to(tdt).cuda()
+    af.step_wait_timeouts(reset=True)
+
+    def launch(work, k, registers, few):
+        out, freg = din.clone(), torch.zeros((P, 4, nc, n), dtype=torch.float64, device="cuda") if registers else None
+        m = len(work) // 64
+        for i in range(0, m, few or m):
+            w = torch.from_numpy(work[64 * i:64 * min(m, i + (few or m))]).cuda()
+            af.patch_step(cfg, w, w.numel() // 64, din, out, dt, grid.dx, grid.dy, freg, tiling=k)
+        torch.cuda.synchronize()
+        return out.double().cpu().numpy(), None if freg is None else freg.cpu().numpy()
+
+    for k, t in enumerate(af.step_tilings()):
+        if t[3]:
+            continue
+        work = af.build_step_work(cfg, np.arange(P), nbr=nbr, tiling=k)
+        assert len(work) // 64 > 152
+        for registers in (True, False):
+            got, freg = launch(work, k, registers, 0)
+            g = cut(got[sample]) if ghosts == "neighbours" else got[sample].reshape(ref.shape)
+            r = cut(ref.reshape(len(sample), -1)) if ghosts == "neighbours" else ref
+            for comp in range(nc):
+                gg, rr = g.reshape(len(sample), nc, -1)[:, comp], r.reshape(len(sample), nc, -1)[:, comp]
+                assert np.nanmax(np.abs(gg - rr)) / np.nanmax(np.abs(rr)) < TOL[prec], (k, registers, comp)
+            if registers:
+                for comp in range(nc):
+                    assert np.abs(freg[sample][:, :, comp] - fref[:, :, comp]).max() < TOL[prec] * np.abs(fref).max(), (k, comp)
+            again, freg2 = launch(work, k, registers, 61)
+            if ghosts == "neighbours":
+                got, again = cut(got), cut(again)
+            assert np.array_equal(got, again, equal_nan=True) and (freg is None or np.array_equal(freg, freg2)), (k, registers)
+    assert af.step_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("eq,n,k", [(1, 32, 3), (0, 32, 3), (1, 32, 0), (1, 16, 4), (0, 16, 4), (1, 18, 6), (0, 18, 7),
+                                    (1, 10, 8), (1, 16, 9)])
+def test_bulk_staging_equals_elementwise_staging_of_many_tiles(af, prec, eq, n, k):
+    """Row bands whose windows are staged in bulk, and bands that start on rows
+    of another 16-byte phase and are staged element by element, give the same
+    step bit for bit, in launches that are not cut further; one agrees with
+    the oracle (test_many_tiles_match_oracle_and_equal_few has the others)."""
+    from paper_2205_07572_gb300.uniform import UniformRun
+    nc = 1 if eq == 0 else 3
+    grid = S.UniformGrid(S.Layout(n, nc), MANY, MANY)
+    own = S.random_owned(grid, seed=90 + n + eq)
+    pst = S.pack_owned(grid, own.astype(np.float32).astype(np.float64) if prec else own)
+    dt = _dt(eq, 0.45, grid.dx, grid.dy, 0.9, -0.4, 1.0)
+    cfg = af.config(eq, prec, n, 0.9, -0.4, 1.0)
+    run = UniformRun(cfg, MANY, MANY, grid.dx, grid.dy, dt, state=np.nan_to_num(pst), tiling=k)
+    tmy, whole = af.step_tilings()[k][1], run.work.cpu().numpy()
+    odd = [0] + list(range(tmy - 3, n, tmy)) + [n]            # starts 0 (bulk), tmy-3, ... (element-wise)
+    four = [0] + list(range(4, n, tmy)) + [n]                 # every start a multiple of 4: all bulk
+    af.step_wait_timeouts(reset=True)
+    outs = []
+    for work in (whole, _resplit(whole, n, odd), _resplit(whole, n, four)):
+        assert len(work) // 64 > 152
+        dout = run.a.clone()
+        af.patch_step(cfg, torch.from_numpy(work).cuda(), len(work) // 64, run.a, dout, dt, grid.dx, grid.dy, tiling=k)
+        torch.cuda.synchronize()
+        outs.append(S.unpack_owned(grid, np.nan_to_num(dout.cpu().numpy()).astype(np.float64).reshape(pst.shape)))
+    assert all(np.array_equal(outs[0][c], o[c]) for o in outs[1:] for c in range(nc))
+    ref = S.unpack_owned(grid, O.run_uniform(O.cfg(eq, n, grid.dx, grid.dy, dt, 0.9, -0.4, 1.0), MANY, MANY, 1, pst))
+    for c in range(nc):
+        assert np.abs(outs[0][c] - ref[c]).max() / np.abs(ref[c]).max() < TOL[prec], c
+    assert af.step_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("eq", [0, 1])
+@pytest.mark.parametrize("neighbours", [False, True])
+def test_whole_patch_bulk_staging_equals_elementwise_staging_of_many_patches(af, eq, neighbours):
+    """169 FP32 patches of 16 x 16 cells that advance their first ghost layer:
+    the 18 x 18 tilings stage whole lattices in bulk, the 18 x 10 tiling element
+    by element; the same bits, in the flux registers too."""
+    n, P, nc = 16, MANY * MANY, 1 if eq == 0 else 3
+    st = S.random_state(S.Layout(n, nc), P, seed=322).astype(np.float32).reshape(P, -1)
+    cfg = af.config(eq, af.F32, n, 0.9, -0.4, 1.0)
+    nbr = None
+    if neighbours:
+        nbr = np.full((P, 8), -1, np.int32)
+        nbr[:, 0], nbr[:, 1] = (np.arange(P) - 1) % P, (np.arange(P) + 1) % P
+        nbr[::7, 1] = -1
+    tl = [t[:3] for t in af.step_tilings()]
+    outs = []
+    af.step_wait_timeouts(reset=True)
+    for k in (tl.index((18, 10, 192)), tl.index((18, 18, 256)), tl.index((18, 18, 128))):
+        work = af.build_step_work(cfg, np.arange(P), nbr=nbr, tiling=k)
+        assert len(work) // 64 > 152
+        din = torch.from_numpy(st).cuda()
+        dout, freg = din.clone(), torch.zeros((P, 4, nc, n), dtype=torch.float64, device="cuda")
+        af.patch_step(cfg, torch.from_numpy(work).cuda(), len(work) // 64, din, dout, 0.4 / n, 1.0 / n, 1.0 / n, freg, tiling=k)
+        torch.cuda.synchronize()
+        outs.append((dout.cpu().numpy(), freg.cpu().numpy()))
+    for o in outs[1:]:
+        assert np.array_equal(o[0], outs[0][0]) and np.array_equal(o[1], outs[0][1])
+    assert af.step_wait_timeouts() == 0
