@@ -91,9 +91,9 @@ struct SC {
     T s, c, n;
 };
 
-// How a displacement's angle z = 2 pi d is turned into sin z and cos z - 1: by
-// their Taylor series up to |z| <= 0.02 (kTiny), 0.25 (kSmall) -- the terms
-// left out are below 5e-8 of sin z and 1e-8 in cos z (FP32; 1e-17, 1e-18 in
+// How a displacement's angle z = 2 pi d is turned into sin z and cos z: by their
+// Taylor series up to |z| <= 0.02 (kTiny), 0.25 (kSmall) -- the terms left out are
+// below 5e-8 of sin z and 1e-8 in cos z (FP32; 1e-17, 1e-18 in
 // FP64), 1e-9 and 7e-9 for kTiny -- and by sincospi beyond.  The host picks by
 // the time step, which bounds d: a 4096-cell run turns by at most 7e-4, a
 // 64-cell run by 0.04.
