@@ -39,7 +39,10 @@ inline int resident_ctas(int threads, size_t smem) {
     static std::atomic<int> held{0};
     int r = held.load(std::memory_order_relaxed);
     if (r == 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, Kern, threads, smem) != cudaSuccess) r = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, Kern, threads, smem) != cudaSuccess) {
+            cudaGetLastError();  // not the launch's error
+            r = 0;
+        }
         held.store(r, std::memory_order_relaxed);
     }
     return r;
