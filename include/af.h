@@ -119,8 +119,8 @@ af_status af_build_step_work(const af_config *cfg, int32_t npatch, const int32_t
  * its interior plus first ghost layer) into near-equal tiles of at most
  * tile_x x tile_y cells, each advanced by one CTA of `threads` threads;
  * persistent = CTAs loop over tiles with the next tile's copies in flight;
- * af_patch_step* refuse persistent tilings (AF_ERR_UNIMPLEMENTED: the kernel
- * is withdrawn), af_patch_step_var runs them as one tile per CTA.  Which is
+ * af_patch_step* refuse persistent tilings (AF_ERR_UNIMPLEMENTED: there is no
+ * such kernel), af_patch_step_var runs them as one tile per CTA.  Which is
  * fastest depends on the patch size, equation and precision; the autotuner
  * (paper_2205_07572_gb300/tune.py) times them. */
 typedef struct {
@@ -249,7 +249,9 @@ af_status af_unpack_owned(const af_config *cfg, int32_t npatch, const void *d_ow
  * d_a, d_b, dt0, dx0, dy0, d_flux_reg as for af_patch_step (d_in, d_out).
  * h_state should be pinned; it and all buffers must stay valid until `stream`
  * has reached this point.  AF_ERR_ARG on NULL pointers, nband < 1 or a band
- * with p0 < 0 or p1 <= p0, else as af_patch_step_tiled and af_pack_owned. */
+ * with p0 < 0 or p1 <= p0, else as af_patch_step_tiled and af_pack_owned: a step
+ * whose arguments are refused enqueues nothing, and after a later error what was
+ * enqueued is ordered before `stream` all the same (the state is then undefined). */
 typedef struct {
     int32_t p0, p1;
     int32_t nwork;
